@@ -145,9 +145,12 @@ soptx_status soptx_mesh_path(soptx_mesh mesh, soptx_path *path);
  *                  element matrices (cached, or one shared matrix), 2
  *                  per-call contraction of the reference integrals in FP32
  *                  (FP32 element matrices of affine cells: k_contract_pairs
- *                  in 2D, k_contract_rows in 3D), 3 node pairs over the
- *                  cached FP64 element matrices (2D affine cells:
- *                  k_contract_pairs reading each pair's blocks once)
+ *                  in 2D, k_block_rows in 3D), 3 node pairs over cached FP64
+ *                  element matrices (2D affine cells: k_contract_pairs) or
+ *                  over the one matrix of a uniform mesh (k_contract_pairs in
+ *                  2D, k_block_rows in 3D), 4 node pairs over the cached
+ *                  element matrices of 3D cells, laid down in the kernel's
+ *                  order (k_block_rows)
  *   *sensitivity : 0 box lattice (Walsh sectors), 1 fused into the row
  *                  gather, 2 strain energy at quadrature points
  *                  (k_strain_energy: affine cells)
@@ -166,7 +169,7 @@ soptx_status soptx_mesh_device_bytes(soptx_mesh mesh, int64_t *bytes);
  * absolute element contributions of the exact value (FP64 element matrices).
  * The order depends on the path: on a general mesh each value is the sum of
  * its element contributions in ascending element order (float-pair
- * accumulation); on a box lattice it is the reference block entry times a
+ * accumulation), on a 3D mesh in up to 32 such shares added in a fixed tree; on a box lattice it is the reference block entry times a
  * signed sum of the (at most 2^d) moduli of the cells the two nodes share,
  * formed by per-axis sums and differences.
  */
@@ -186,15 +189,13 @@ soptx_status soptx_sensitivity(soptx_mesh mesh, const double *d_rho, const doubl
 /* One pass that produces both K(rho) and the sensitivities (the per-iteration
  * step); same arguments and results as the two calls above: K and dc bitwise,
  * c the same fixed-order sum of block partials (on 2D meshes of affine cells
- * other than box lattices over one block per SM, so its last bits may differ
- * from the separate call's when the mesh has more cells than the SMs' blocks
- * hold).  On a 2D box lattice the sensitivities run on a second, mesh-owned
- * stream beside the assembly; on other 2D meshes of affine cells they run
- * first on that stream (created at the highest stream priority), one block per
- * SM, beside the assembly on `stream`; on 3D meshes of affine cells the
- * assembly runs on that stream beside the sensitivities on `stream` (the
- * stream and two events are made by the first such call); everything is
- * ordered on `stream` when the call returns. */
+ * other than box lattices, and 3D ones, over a few blocks per SM, so its last
+ * bits may differ from the separate call's when the mesh has more cells than
+ * those blocks hold).  On a 2D box lattice the sensitivities run on a second, mesh-owned
+ * stream beside the assembly; on other meshes they run first on that stream
+ * (created at the highest stream priority), a few blocks per SM, beside the
+ * assembly on `stream` (the stream and two events are made by the first such
+ * call); everything is ordered on `stream` when the call returns. */
 soptx_status soptx_assemble_and_sensitivity(soptx_mesh mesh, const double *d_rho,
                                             const double *d_u, double *d_vals,
                                             double *d_dc, double *d_c, void *stream);
@@ -312,9 +313,10 @@ soptx_status soptx_host_plan(int dim, soptx_cell cell, int order, int64_t n_vert
 /*
  * Host-only inspection (no device work, usable without a GPU) of the node-pair
  * schedule by which the pair kernel forms K(rho) = sum_e E(rho_e) K_e^0
- * (Sec. 2.2) on 2D affine meshes and uniform meshes.  Built exactly as
- * soptx_mesh_create builds it for a mesh; the mesh arguments are those of
- * soptx_host_plan.
+ * (Sec. 2.2) on 2D affine meshes and 2D uniform meshes.  Built exactly as
+ * soptx_mesh_create builds it for a 2D mesh (3D meshes are assembled by
+ * another kernel; their tables are built for inspection only); the mesh
+ * arguments are those of soptx_host_plan.
  *
  * A pair is two nodes a, b that share a cell (or a = b).  In 2D K is
  * symmetric, so each unordered pair appears once, owned by whichever node
@@ -348,11 +350,11 @@ soptx_status soptx_host_pair_tables(int dim, soptx_cell cell, int order, int64_t
                                     uint32_t *pair_meta, int32_t *record_cell, uint16_t *record_pair);
 
 /*
- * Host-only inspection (no device work, usable without a GPU) of the
- * node-owner schedule by which 3D meshes with FP32 element matrices form
- * K(rho) = sum_e E(rho_e) K_e^0 (Sec. 2.2): a group of nb lanes owns the d rows
- * of one node and walks the node's cells as a chain.  Built exactly as
- * soptx_mesh_create builds it; the mesh arguments are those of soptx_host_plan.
+ * Host-only inspection (no device work, usable without a GPU) of a node-owner
+ * schedule of K(rho) = sum_e E(rho_e) K_e^0 (Sec. 2.2) on 3D meshes: a group of
+ * nb lanes owns the d rows of one node and walks the node's cells as a chain.
+ * No kernel of the library walks it (3D meshes are assembled by chunks of
+ * complete rows); the mesh arguments are those of soptx_host_plan.
  *   node_records int32 [n_nodes][4], in processing order (cell count
  *     descending, then node id): the node's first row block offset (low and
  *     high 32-bit words; the value index of its entry (d n, .) is d^2 times

@@ -37,7 +37,7 @@ static void free_device(DeviceMesh &d)
                     d.pos, d.geo, d.M, d.K, d.scratch, d.Edf, d.kappa, d.K0, d.sectors, d.udf, d.part,
                     d.inc_e, d.inc_a, d.counter, d.xcell, d.qw, d.qdphi, d.qdgeo, d.cg, d.lat_bad, d.stage,
                     d.kvals, d.sgeo, d.sq, d.ssf, d.cgeo, d.Mf, d.ptoff, d.pia, d.pib, d.pmeta, d.pre, d.prm, d.pblk,
-                    d.cnrec, d.cinc_e, d.cinc_a, d.crec, d.cticket};
+                    d.bblob, d.bcoff, d.bcell, d.bM, d.bkblk, d.cticket};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (d.cg_exec) cudaGraphExecDestroy(d.cg_exec);
@@ -117,10 +117,10 @@ static soptx_status setup_strain(soptx_mesh_s &m, const RefElement &ref, cudaStr
     for (size_t t = 0; t < q.dphi.size(); t++) tab[q.nq + t] = split_pair(q.dphi[t]);
     const int ng = h.dim * h.dim + 1;
     const int64_t ncg = m.path == SOPTX_PATH_UNIFORM ? 1 : h.nc;
-    std::vector<float2> sg((size_t)ncg * ng);
+    std::vector<float2> sg(h.nonaffine ? 0 : (size_t)ncg * ng);
     for (size_t t = 0; t < sg.size(); t++) sg[t] = split_pair(h.geo[t]);
     soptx_status s = upload(&m.d.sq, tab, st, m.device_bytes, "quadrature table");
-    if (s == SOPTX_OK) s = upload(&m.d.sgeo, sg, st, m.device_bytes, "cell geometry pairs");
+    if (s == SOPTX_OK && !h.nonaffine) s = upload(&m.d.sgeo, sg, st, m.device_bytes, "cell geometry pairs");
     if (s == SOPTX_OK && h.dim == 3 && !is_simplex(h.cell) && (h.order == 2 || h.order == 3)) {
         // the 1D factors of the tensor rule, for the sum-factorised kernel
         std::vector<double> w1, val, der;
@@ -136,10 +136,20 @@ static soptx_status setup_strain(soptx_mesh_s &m, const RefElement &ref, cudaStr
         }
         s = upload(&m.d.ssf, sf, st, m.device_bytes, "1D factors of the rule");
     }
-    if (s == SOPTX_OK) {
-        m.d.snq = q.nq;
-        m.d.strain = true;
+    m.d.snq = q.nq;
+    if (s == SOPTX_OK && h.nonaffine) {
+        // general cells: the geometry of every point, computed on the device
+        const size_t bytes = (size_t)h.nc * q.nq * ng * sizeof(float2);
+        cudaError_t e = dev_alloc((void **)&m.d.sgeo, bytes);
+        if (e == cudaSuccess) e = launch_point_geometry(m, st);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            s = cuda_status(e, "point geometry");
+        } else {
+            m.device_bytes += (int64_t)bytes;
+        }
     }
+    if (s == SOPTX_OK) m.d.strain = true;
     return s;
 }
 
@@ -159,9 +169,8 @@ static soptx_status setup_strain(soptx_mesh_s &m, const RefElement &ref, cudaStr
 // The same tables serve the cached FP64 element matrices of 2D cells (cached:
 // each record's 2 x 2 block is also gathered into record order) and the one
 // FP64 matrix of a uniform mesh (unif); for those the local pair is stored as
-// a_loc << 8 | b_loc.  In 3D (uniform meshes) every node takes all of its own
-// column blocks instead of the pairs after it, so no block is written
-// transposed.
+// a_loc << 8 | b_loc.  In 3D (soptx_host_pair_tables only; blockrows.cu assembles
+// 3D meshes) every node takes all of its own column blocks instead.
 static constexpr size_t kPairWindow = 4096;
 
 struct PairTables {
@@ -357,8 +366,8 @@ static soptx_status setup_contract_pairs(soptx_mesh_s &m, const RefElement &ref,
     return s;
 }
 
-// Tables of the node-owner contraction of 3D cells (k_contract_rows), on the
-// host.  False when a node meets 65536 cells or more (a node record holds the
+// The node-owner schedule of 3D cells (soptx_host_row_tables), on the host; no
+// kernel walks it any more (blockrows.cu assembles 3D meshes).  False when a node meets 65536 cells or more (a node record holds the
 // incident-cell count in 16 bits): such fans keep the cached gather.
 struct RowTables {
     // per node in processing order: its row block offset (node_off, low and
@@ -483,38 +492,87 @@ static bool build_row_tables(const HostMesh &h, RowTables &T)
     return true;
 }
 
-static soptx_status setup_contract_rows(soptx_mesh_s &m, const RefElement &ref, cudaStream_t st)
+// Tables of the block-row kernel of 3D meshes (blockrows.cu).  The mesh keeps the
+// cached gather when its largest node does not fit in the tables or in shared memory.
+static soptx_status setup_block_rows(soptx_mesh_s &m, const RefElement &ref, const double *coords, const int32_t *cv,
+                                     int src, cudaStream_t st)
 {
     const HostMesh &h = m.h;
-    const int d = h.dim, nb = h.nb, ng = d * d + 1, n4 = d == 3 ? 3 : 2, mp = d == 3 ? 12 : 4;
-    RowTables T;
-    if (!build_row_tables(h, T)) return SOPTX_OK;
-    std::vector<float4> cg((size_t)h.nc * n4, make_float4(0.f, 0.f, 0.f, 0.f));
-    for (int64_t e = 0; e < h.nc; e++) {
-        float *dst = reinterpret_cast<float *>(&cg[(size_t)e * n4]);
-        for (int t = 0; t < ng; t++) dst[t] = (float)h.geo[(size_t)e * ng + t];
+    const int nb = h.nb;
+    std::vector<float> mf;
+    std::vector<float4> cell, blk;
+    if (src == kBlockContract) {
+        mf.assign((size_t)nb * nb * 12, 0.f);
+        for (int a = 0; a < nb; a++)
+            for (int b = 0; b < nb; b++)
+                for (int kl = 0; kl < 9; kl++)
+                    mf[((size_t)a * nb + b) * 12 + kl] = (float)ref.M[((size_t)kl * nb + a) * nb + b];
     }
-    std::vector<float> mf((size_t)nb * nb * mp, 0.f);
-    for (int a = 0; a < nb; a++)
-        for (int b = 0; b < nb; b++)
-            for (int k = 0; k < d; k++)
-                for (int l = 0; l < d; l++)
-                    mf[((size_t)a * nb + b) * mp + k * d + l] = (float)ref.M[(((size_t)k * d + l) * nb + a) * nb + b];
-    soptx_status s = upload(&m.d.cgeo, cg, st, m.device_bytes, "cell geometry");
-    if (s == SOPTX_OK) s = upload(&m.d.Mf, mf, st, m.device_bytes, "reference integrals (FP32)");
-    if (s == SOPTX_OK) s = upload(&m.d.cnrec, T.nrec, st, m.device_bytes, "node records");
-    if (s == SOPTX_OK) s = upload(&m.d.cinc_e, T.ce, st, m.device_bytes, "contraction cell chains");
-    if (s == SOPTX_OK) s = upload(&m.d.cinc_a, T.ca, st, m.device_bytes, "contraction local indices");
-    if (s == SOPTX_OK) s = upload(&m.d.crec, T.rec, st, m.device_bytes, "contraction lane records");
-    if (s == SOPTX_OK) s = upload(&m.d.cticket, std::vector<unsigned>(2, 0u), st, m.device_bytes, "round counter");
-    if (s == SOPTX_OK) m.d.contract = true;
+    BlockLimits L;
+    // FP32 blocks are symmetric only to their rounding: each is formed for its own place
+    L.sym = m.prec == SOPTX_ELEM_FP64;
+    // lanes that read the same block of K^0 beside one another (Q3 box 26x9x9: 202 -> 197 us)
+    L.by_code = src == kBlockUniform;
+    BlockTables T;
+    if (!build_block_tables(h, coords, cv, L, T)) return SOPTX_OK;
+    const int64_t smem = block_smem(src, nb, T);
+    if (smem > 220 * 1024) return SOPTX_OK;
+    soptx_status s = SOPTX_OK;
+    if (src == kBlockContract) {
+        cell.assign((size_t)h.nc * 3, make_float4(0.f, 0.f, 0.f, 0.f));
+        for (int64_t e = 0; e < h.nc; e++)
+            for (int t = 0; t < 10; t++)
+                reinterpret_cast<float *>(&cell[(size_t)e * 3])[t] = (float)h.geo[(size_t)e * 10 + t];
+    } else if (src == kBlockUniform) {
+        // the blocks of the one element matrix, each five float4s of two pairs
+        const int ld = h.ldof;
+        std::vector<float2> K((size_t)ld * ld);
+        blk.assign((size_t)nb * nb * 5, make_float4(0.f, 0.f, 0.f, 0.f));
+        if (m.prec == SOPTX_ELEM_FP32) {
+            std::vector<float> Kf(K.size());
+            s = cuda_status(cudaMemcpy(Kf.data(), m.d.K, Kf.size() * sizeof(float), cudaMemcpyDeviceToHost), "K0");
+            for (size_t q = 0; q < K.size(); q++) K[q] = make_float2(Kf[q], 0.f);
+        } else {
+            s = cuda_status(cudaMemcpy(K.data(), m.d.K, K.size() * sizeof(float2), cudaMemcpyDeviceToHost), "K0");
+        }
+        for (int a = 0; a < nb; a++)
+            for (int b = 0; b < nb; b++)
+                for (int p = 0; p < 9; p++)
+                    reinterpret_cast<float2 *>(&blk[((size_t)a * nb + b) * 5])[p] =
+                        K[(size_t)(3 * a + p / 3) * ld + 3 * b + p % 3];
+    }
+    if (s == SOPTX_OK && !cell.empty()) s = upload(&m.d.bcell, cell, st, m.device_bytes, "cell geometry");
+    if (s == SOPTX_OK && !mf.empty()) s = upload(&m.d.bM, mf, st, m.device_bytes, "reference integrals (FP32)");
+    if (s == SOPTX_OK && !blk.empty()) s = upload(&m.d.bkblk, blk, st, m.device_bytes, "element matrix blocks");
+    if (s == SOPTX_OK) {
+        uint32_t *p = nullptr;   // (32-bit words, a whole number of 16-byte units)
+        s = upload(&p, T.blob, st, m.device_bytes, "chunk records");
+        m.d.bblob = reinterpret_cast<uint4 *>(p);
+    }
+    if (s == SOPTX_OK) s = upload(&m.d.bcoff, T.coff, st, m.device_bytes, "chunk offsets");
+    if (s == SOPTX_OK) s = upload(&m.d.cticket, std::vector<unsigned>(4, 0u), st, m.device_bytes, "chunk counter");
+    m.d.bcell_bits = T.cell_bits;
+    m.d.bmax_blob = T.max_blob;
+    m.d.bmax_cells = T.max_cells;
+    m.d.bmax_stage = T.max_stage;
+    m.d.bmax_rows = T.max_rows;
+    m.d.bsmem = (int)smem;
+    m.d.bsrc = src;
+    if (s == SOPTX_OK) m.d.bchunks = T.nchunks;
+    if (s == SOPTX_OK && src == kBlockStream) {
+        const int64_t bytes = std::max<int64_t>(T.rows, 1) * block_row_bytes();
+        cudaError_t e = dev_alloc((void **)&m.d.bkblk, (size_t)bytes);
+        if (e == cudaSuccess) e = launch_block_stream(m, st);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            s = cuda_status(e, "streamed element blocks");
+        } else {
+            m.device_bytes += bytes;
+        }
+    }
+    // (the host tables go out of scope: their copies have to be done)
+    if (s == SOPTX_OK) s = cuda_status(cudaStreamSynchronize(st), "chunk records");
     return s;
-}
-
-// FP32 element matrices of affine cells: the tables of the per-call contraction.
-static soptx_status setup_contract(soptx_mesh_s &m, const RefElement &ref, cudaStream_t st)
-{
-    return m.h.dim == 2 ? setup_contract_pairs(m, ref, st, false) : setup_contract_rows(m, ref, st);
 }
 
 static bool material_ok(const soptx_material *m, int dim, Material &out, std::string &err)
@@ -702,26 +760,35 @@ soptx_status soptx_mesh_create(int dim, soptx_cell cell, int order, int64_t n_ve
         }
         if (s == SOPTX_OK) s = cuda_status(cudaStreamSynchronize(st), "mesh setup");
     }
-    if (s == SOPTX_OK && m->path != SOPTX_PATH_LATTICE && !h.nonaffine && h.nc > 0) {
+    if (s == SOPTX_OK && m->path != SOPTX_PATH_LATTICE && h.nc > 0 && (!h.nonaffine || prec == SOPTX_ELEM_FP64)) {
         // affine cells off the lattice: the sensitivities from the strain energy at
         // the points of a rule exact for it (G and |det J| per cell as float pairs,
-        // the weights and reference gradients of the rule)
+        // the weights and reference gradients of the rule); general cells at the
+        // points of the rule that defines their FP64 element matrices (FP32 ones keep
+        // the gather: their sensitivities are those of the rounded matrices)
         s = setup_strain(*m, ref, st);
-        // FP32 element matrices: the assembly contracts the reference integrals with
-        // each cell's Jacobian per call (FP32 tables), the cache is not read
-        if (s == SOPTX_OK && prec == SOPTX_ELEM_FP32 && m->path == SOPTX_PATH_CACHED &&
-            contract_fits(h.dim, h.nb, h.max_deg))
-            s = setup_contract(*m, ref, st);
-        // FP64 element matrices of 2D cells: the pair kernel reads each node pair's
-        // blocks of the cache once for both row blocks
-        if (s == SOPTX_OK && prec == SOPTX_ELEM_FP64 && m->path == SOPTX_PATH_CACHED && h.dim == 2 &&
-            contract_fits(h.dim, h.nb, h.max_deg))
-            s = setup_contract_pairs(*m, ref, st, true);
-        // FP64 element matrix of a uniform mesh (boxes of order 2 and 3): the pair
-        // kernel reads its blocks through L1
-        if (s == SOPTX_OK && prec == SOPTX_ELEM_FP64 && m->path == SOPTX_PATH_UNIFORM &&
+        // 2D: FP32 element matrices contracted per call, the cache not read; FP64 ones
+        // and a uniform mesh's one matrix: the pair kernel reads each node pair's
+        // blocks once for both row blocks
+        if (s == SOPTX_OK && h.dim == 2 && m->path == SOPTX_PATH_CACHED && !h.nonaffine && contract_fits(h.dim, h.nb, h.max_deg))
+            s = setup_contract_pairs(*m, ref, st, prec == SOPTX_ELEM_FP64);
+        if (s == SOPTX_OK && h.dim == 2 && prec == SOPTX_ELEM_FP64 && m->path == SOPTX_PATH_UNIFORM &&
             pairs_fit(h.dim, h.nb, h.max_deg))
             s = setup_contract_pairs(*m, ref, st, false, true);
+    }
+    if (s == SOPTX_OK && m->path != SOPTX_PATH_LATTICE && h.dim == 3 && h.nc > 0 &&
+        (!h.nonaffine || prec == SOPTX_ELEM_FP64)) {
+        // 3D: the block rows of one matrix for all cells, of FP32 matrices of affine
+        // cells contracted per call, or of the cached matrices
+        const int src = m->path == SOPTX_PATH_UNIFORM                   ? kBlockUniform
+                        : prec == SOPTX_ELEM_FP32          ? kBlockContract
+                                                                  : kBlockStream;
+        try {
+            s = setup_block_rows(*m, ref, coords, cell_vertices, src, st);
+        } catch (const std::bad_alloc &) {
+            set_error("host allocation failed building the chunk records");
+            s = SOPTX_ENOMEM;
+        }
     }
     if (s == SOPTX_OK && (m->path != SOPTX_PATH_LATTICE || !d.sectors)) {
         // per-call float-pair moduli and displacements, per-(cell, node) partials
@@ -924,7 +991,14 @@ soptx_status soptx_mesh_routes(soptx_mesh m, int32_t *assembly, int32_t *sensiti
 {
     if (!m) SOPTX_FAIL(SOPTX_EINVAL, "mesh is NULL");
     if (assembly)
-        *assembly = m->path == SOPTX_PATH_LATTICE ? 0 : m->d.contract ? 2 : (m->d.pcached || m->d.puniform) ? 3 : 1;
+        {
+        const auto &d = m->d;
+        *assembly = m->path == SOPTX_PATH_LATTICE                                                   ? 0
+                    : d.contract || (d.bchunks >= 0 && d.bsrc == kBlockContract)                ? 2
+                    : d.pcached || d.puniform || (d.bchunks >= 0 && d.bsrc == kBlockUniform) ? 3
+                    : d.bchunks >= 0                                                            ? 4
+                                                                                                : 1;
+    }
     if (sensitivity) *sensitivity = (m->path == SOPTX_PATH_LATTICE && m->d.sectors) ? 0 : (m->d.strain ? 2 : 1);
     return SOPTX_OK;
 }

@@ -22,20 +22,8 @@
 //                    The same kernel reads the blocks instead for the cached
 //                    FP64 element matrices of 2D affine cells (each record's
 //                    block gathered into record order at mesh creation) and
-//                    for the one FP64 matrix of a uniform mesh (boxes of order
-//                    2 and 3; in 3D each node then assembles all of its own
-//                    rows, no transposed writes).
-//  k_contract_rows : the same blocks for 3D cells, with the rows of one node
-//                    owned by a group of nb lanes (nb = basis functions per
-//                    cell) that walks the node's incident cells as a chain
-//                    fixed at mesh creation (each next cell shares as many of
-//                    the lanes' current column nodes as possible); lane b takes
-//                    the cell's local node b and adds E_e K into the rows'
-//                    float-pair accumulators in shared memory, keeping them in
-//                    registers while its column block continues into the next
-//                    cell.  (The pair layout in 3D writes every transposed
-//                    block as three scattered 24-byte row pieces; the L2 then
-//                    writes partly filled sectors back and fetches them again.)
+//                    for the one FP64 matrix of a 2D uniform mesh (boxes of
+//                    order 2 and 3).  3D meshes: blockrows.cu.
 //  k_strain_energy : s_e = u_e^T K_e^0 u_e = int_e lam (div u)^2 + 2 mu eps:eps
 //                    by a quadrature rule exact for the energy density of the
 //                    cell's order, one thread per cell: the reference
@@ -95,26 +83,6 @@ struct PairArgs {
     float lam, mu;
     double *__restrict__ vals;
 };
-
-// The node-owner contraction of 3D cells (k_contract_rows).
-struct ContractArgs {
-    int64_t nn;
-    int max_deg;
-    const int4 *__restrict__ nrec;       // per processing position: row block offset, q0, cnt << 16 | deg
-    unsigned *__restrict__ ticket;       // [0] rounds handed out, [1] warps done (both zero between calls)
-    const int32_t *__restrict__ inc_e;   // each node's cells in chain order
-    const uint8_t *__restrict__ inc_a;   // the node's local index in each
-    const uint16_t *__restrict__ rec;    // per (incidence, lane): column block p (bits 0-8), local node b
-                                         // (9-13), first (14) / last (15) meeting of the block
-    const float4 *__restrict__ cgeo;
-    const float *__restrict__ Mf;
-    const float2 *__restrict__ Edf;
-    const double *__restrict__ rho;
-    SimpParams sp;
-    float lam, mu;
-    double *__restrict__ vals;
-};
-
 
 template <int D>
 __device__ __forceinline__ void contract_block(const float *M, const float *G, float det, float lam, float mu,
@@ -188,273 +156,6 @@ __device__ __forceinline__ void acc_add(float &s, float &c, df x)
     two_sum(s, x.h, t, err);
     s = t;
     c = __fadd_rn(c, __fadd_rn(x.l, err));
-}
-
-// Plain-FP64 redo of one node by its group (a modulus outside the float-pair
-// range): the same FP32 blocks times E(rho_e) in FP64, summed in ascending
-// cell order into acc (as doubles), then stored.
-template <int D, int NB>
-__device__ __noinline__ void contract_node_fp64(const ContractArgs &A, const float *Ms, unsigned gmask, int b,
-                                                int64_t off, int deg, int32_t q0, int32_t cnt, double *acc)
-{
-    const int rowlen = D * deg, blk = D * rowlen;
-    for (int t = b; t < blk; t += NB) acc[t] = 0.0;
-    __syncwarp(gmask);
-    for (int32_t t = 0; t < cnt; t++) {
-        const int32_t q = q0 + t;
-        const int64_t e = A.inc_e[q];
-        const int a = A.inc_a[q];
-        const uint32_t r = A.rec[(int64_t)q * NB + b];
-        const int p = (int)(r & 511u), lb = (int)((r >> 9) & 31u);
-        float G[D * D], det, M[D * D], K[D][D];
-        load_cgeo<D>(A.cgeo, e, G, det);
-        load_mpair<D>(Ms, a * NB + lb, M);
-        contract_block<D>(M, G, det, A.lam, A.mu, K);
-        const double E = simp_E(A.sp, A.rho[e]);
-#pragma unroll
-        for (int i = 0; i < D; i++)
-#pragma unroll
-            for (int j = 0; j < D; j++) acc[i * rowlen + D * p + j] += E * (double)K[i][j];
-        __syncwarp(gmask);
-    }
-    double *out = A.vals + (int64_t)D * D * off;
-    for (int t = b; t < blk; t += NB) __stcs(out + t, acc[t]);
-    __syncwarp(gmask);
-}
-
-// NPW = 32 / NB nodes per warp, NB lanes each; lanes beyond NPW NB idle.
-template <int D, int NB, int MINB>
-__global__ void __launch_bounds__(256, MINB) k_contract_rows(const ContractArgs A)
-{
-    static_assert(D == 3, "the node-owner contraction serves 3D cells");
-    constexpr int NPW = 32 / NB;
-    constexpr int MP = MPad<D>::n;
-    constexpr int G4 = CGeo<D>::n4;
-    extern __shared__ float4 csm4[];
-    float *Ms = reinterpret_cast<float *>(csm4);
-    float2 *accs = reinterpret_cast<float2 *>(Ms + NB * NB * MP);
-    for (int t = threadIdx.x; t < NB * NB * MP; t += blockDim.x) Ms[t] = A.Mf[t];
-    __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
-    const int g = lane / NB, b = lane - g * NB;
-    const bool act = g < NPW;
-    const int gg = act ? g : NPW - 1;
-    const unsigned gmask = (NB == 32 ? kFull : ((1u << NB) - 1u)) << (gg * NB);
-    const int acc_len = D * D * A.max_deg;
-    const int gacc = (warp * NPW + gg) * acc_len;   // the group's accumulators: accs[gacc ...]
-    // Round r takes positions r NPW .. r NPW + NPW - 1 of the processing order
-    // (nodes by incident-cell count, largest first), so a warp's groups walk
-    // about as many cells each.  Warps take rounds from a counter, three ahead
-    // (the prefetch below reaches two rounds past the current one), so a CTA
-    // that starts late, beside another kernel, simply takes fewer.  The last warp
-    // to finish sets the counter back to zero.  A node's record is one 16-byte load.
-    const int64_t rounds = (A.nn + NPW - 1) / NPW;
-    auto grab = [&]() -> int64_t {
-        unsigned t = 0;
-        if (lane == 0) t = atomicAdd(A.ticket, 1u);
-        return (int64_t)__shfl_sync(kFull, t, 0);
-    };
-    struct Node {
-        int64_t off;
-        int32_t q0, cnt, deg;
-    };
-    auto load_node = [&](int64_t n0, Node &N) {
-        N = Node{0, 0, 0, 0};
-        if (act && n0 + g < A.nn) {
-            const int4 r = __ldg(A.nrec + n0 + g);
-            N.off = (int64_t)(uint32_t)r.x | ((int64_t)r.y << 32);
-            N.q0 = r.z;
-            N.cnt = (int32_t)((uint32_t)r.w >> 16);
-            N.deg = r.w & 0xffff;
-        }
-    };
-    auto warp_max = [](int x) { return (int)__reduce_max_sync(kFull, (unsigned)x); };
-    struct Cell {
-        float4 g[G4];
-        float2 E;
-        int a, p;
-    };
-    // The rounds' incidences form one stream: cell, a and the lane record are
-    // loaded two items ahead, geometry and modulus one ahead, across the end of
-    // a round into the next one (or the one after, when the next has a single
-    // item), so a node's first cells are in flight while the previous node's
-    // rows are written.  Position s counts from the current round's first item;
-    // a group's index past its node's last incidence is clamped to it (the item
-    // is not used), so the loads need no predicates.
-    // the round after next: only its first incidence and cell count
-    auto load_head = [&](int64_t n0, int32_t &q, int32_t &c) {
-        q = 0;
-        c = 0;
-        if (act && n0 + g < A.nn) {
-            const int2 r = __ldg(reinterpret_cast<const int2 *>(A.nrec + n0 + g) + 1);
-            q = r.x;
-            c = (int32_t)((uint32_t)r.y >> 16);
-        }
-    };
-    Node N0, N1;
-    int32_t q02, cnt2;
-    int64_t r0 = grab(), r1 = grab(), r2 = grab();
-    load_node(r0 * NPW, N0);
-    load_node(r1 * NPW, N1);
-    load_head(r2 * NPW, q02, cnt2);
-    int imax0 = warp_max(N0.cnt), imax1 = warp_max(N1.cnt);
-    auto fetch_idx = [&](int s, int32_t &e, int &a, int &p) {
-        int32_t qs = N0.q0, cs = N0.cnt;
-        int k = s;
-        if (s >= imax0) {
-            k = s - imax0;
-            if (k < imax1) {
-                qs = N1.q0;
-                cs = N1.cnt;
-            } else {
-                k -= imax1;
-                qs = q02;
-                cs = cnt2;
-            }
-        }
-        const int32_t q = qs + min(k, max(cs - 1, 0));
-        e = __ldg(A.inc_e + q);
-        a = __ldg(A.inc_a + q);
-        p = __ldg(A.rec + (int64_t)q * NB + b);
-    };
-    auto fetch_data = [&](int32_t e, int a, int p, Cell &c) {
-        const float4 *gp = A.cgeo + (int64_t)G4 * e;
-#pragma unroll
-        for (int w = 0; w < G4; w++) c.g[w] = __ldg(gp + w);
-        c.E = __ldg(A.Edf + e);
-        c.a = a;
-        c.p = p;
-    };
-    int32_t e1, e2;
-    int a1, p1, a2, p2;
-    fetch_idx(0, e1, a1, p1);
-    fetch_idx(1, e2, a2, p2);
-    Cell c0, c1;
-    fetch_data(e1, a1, p1, c0);
-    while (r0 < rounds) {
-        const int64_t n0 = r0 * NPW;
-        const bool has = act && n0 + g < A.nn;
-        const int64_t off = N0.off;
-        const int deg = N0.deg;
-        const int32_t q0 = N0.q0, cnt = N0.cnt;
-        // no zeroing: every block of the rows is met by some cell, and its first
-        // meeting starts the sums from zero
-        double *const out = A.vals + (int64_t)D * D * off;
-        const int rowlen = D * deg, blk = D * rowlen;
-
-        const int ro1 = rowlen, ro2 = 2 * rowlen;
-        bool bad = false;
-        // the lane's row sums of its current column block: read from shared memory
-        // when the block starts, written back when the next cell has another one
-        float2 v[D][D];
-        bool held = false;
-        auto body = [&](const Cell &cur, Cell &nxt, int it) {
-            fetch_data(e2, a2, p2, nxt);
-            fetch_idx(it + 2, e2, a2, p2);
-            if (it < cnt) {
-                bad |= isnan(cur.E.y);
-                float G[D * D], det;
-                if (D == 3) {
-                    G[0] = cur.g[0].x; G[1] = cur.g[0].y; G[2] = cur.g[0].z; G[3] = cur.g[0].w;
-                    G[4] = cur.g[1].x; G[5] = cur.g[1].y; G[6] = cur.g[1].z; G[7] = cur.g[1].w;
-                    G[8] = cur.g[2].x;
-                    det = cur.g[2].y;
-                } else {
-                    G[0] = cur.g[0].x; G[1] = cur.g[0].y; G[2] = cur.g[0].z; G[3] = cur.g[0].w;
-                    det = cur.g[1].x;
-                }
-                const int slot = cur.p & 511, lb = (cur.p >> 9) & 31;
-                float M[D * D], K[D][D];
-                load_mpair<D>(Ms, cur.a * NB + lb, M);
-                contract_block<D>(M, G, det, A.lam, A.mu, K);
-                // the lane's slots are distinct within a cell, and a block held in
-                // registers is no other lane's in the next cell
-                const int base = gacc + D * slot;
-                const int rbase[3] = {base, base + ro1, base + ro2};
-                const bool keep = it + 1 < cnt && (nxt.p & 511) == slot;
-                if (!held) {
-                    if (cur.p & 0x4000) {
-#pragma unroll
-                        for (int i = 0; i < D; i++)
-#pragma unroll
-                            for (int j = 0; j < D; j++) v[i][j] = make_float2(0.f, 0.f);
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < D; i++)
-#pragma unroll
-                            for (int j = 0; j < D; j++) v[i][j] = accs[rbase[i] + j];
-                    }
-                }
-#pragma unroll
-                for (int i = 0; i < D; i++)
-#pragma unroll
-                    for (int j = 0; j < D; j++) {
-                        // E K as a pair: TwoProd of the head, the tail's product
-                        const float k = K[i][j];
-                        const float ph = __fmul_rn(cur.E.x, k);
-                        const float pl = __fmaf_rn(cur.E.y, k, __fmaf_rn(cur.E.x, k, -ph));
-                        acc_add(v[i][j].x, v[i][j].y, df{ph, pl});
-                    }
-                if (!keep) {
-#pragma unroll
-                    for (int i = 0; i < D; i++)
-#pragma unroll
-                        for (int j = 0; j < D; j++) accs[rbase[i] + j] = v[i][j];
-                }
-                held = keep;
-            }
-            __syncwarp();
-        };
-        for (int it = 0; it < imax0; it += 2) {
-            body(c0, c1, it);
-            if (it + 1 < imax0) body(c1, c0, it + 1);
-        }
-        if (imax0 & 1) {
-            // after an odd count the next round's first cell arrived in c1
-            const Cell t = c0;
-            c0 = c1;
-            c1 = t;
-        }
-        // a group whose node met an out-of-range modulus redoes it in FP64
-        const unsigned badm = __ballot_sync(kFull, bad);
-        if (has && (badm & gmask)) {
-            contract_node_fp64<D, NB>(A, Ms, gmask, b, off, deg, q0, cnt, reinterpret_cast<double *>(accs + gacc));
-        } else if (has) {
-            // the rows leave as FP64 values, two per store where the destination is
-            // 16-byte aligned (an odd 8-byte head is stored on its own)
-            const int head = (int)((reinterpret_cast<uintptr_t>(out) >> 3) & 1u);
-            if (head && b == 0) {
-                const float2 v = accs[gacc];
-                __stcs(out, pair_to_double(v.x, v.y));
-            }
-            for (int t = head + 2 * b; t < blk; t += 2 * NB) {
-                const float2 v0 = accs[gacc + t];
-                const double d0 = pair_to_double(v0.x, v0.y);
-                if (t + 1 < blk) {
-                    const float2 v1 = accs[gacc + t + 1];
-                    __stcs(reinterpret_cast<double2 *>(out + t), make_double2(d0, pair_to_double(v1.x, v1.y)));
-                } else {
-                    __stcs(out + t, d0);
-                }
-            }
-        }
-        __syncwarp();
-        r0 = r1;
-        r1 = r2;
-        r2 = grab();
-        N0 = N1;
-        load_node(r1 * NPW, N1);
-        load_head(r2 * NPW, q02, cnt2);
-        imax0 = imax1;
-        imax1 = warp_max(N1.cnt);
-    }
-    if (lane == 0) {
-        __threadfence();
-        if (atomicAdd(A.ticket + 1, 1u) == gridDim.x * (unsigned)wpb - 1u) {
-            A.ticket[0] = 0u;
-            A.ticket[1] = 0u;
-        }
-    }
 }
 
 // Row i of a d x d block of FP64 values at o (row stride rl), and the block's
@@ -913,6 +614,10 @@ struct StrainArgs {
     SimpParams sp;
     const float2 *__restrict__ geo;   // [nc or 1][d*d + 1] G row-major, |det J|, as pairs
     int64_t geo_stride;               // d*d + 1, or 0 when every cell has the same Jacobian
+    // general bilinear / trilinear cells: G and w |det J| at every point, entry t of
+    // point q of cell e at geo[e geo_stride + (q (d*d + 1) + t) geo_step]
+    bool general;
+    int64_t geo_step;
     const float2 *__restrict__ qw;    // [nq] weights
     const float2 *__restrict__ qd;    // [nq][nb][d] reference gradients
     float2 lam, mu;                   // Lame constants at E = 1, as pairs
@@ -928,7 +633,9 @@ struct StrainArgs {
 // <= 256 (the grid sum of c).
 // NBT = the cell's node count, so the staging loads of a cell issue together,
 // or 0 for any count (runtime loops).
-template <int D, bool PAIR, int NBT>
+// GEN: general cells, the geometry of every point read as it is needed (det then
+// holds w |det J|).
+template <int D, bool PAIR, int NBT, bool GEN = false>
 __global__ void __launch_bounds__(128) k_strain_energy(const StrainArgs A)
 {
     using S = SArith<PAIR>;
@@ -966,11 +673,18 @@ __global__ void __launch_bounds__(128) k_strain_energy(const StrainArgs A)
             }
             V G[D * D], det;
             const float2 *gp = A.geo + e * A.geo_stride;
+            auto load_geo = [&]() {
 #pragma unroll
-            for (int t = 0; t < D * D; t++) G[t] = S::from_pair(gp[t]);
-            det = S::from_pair(gp[D * D]);
+                for (int t = 0; t < D * D; t++) G[t] = S::from_pair(gp[t * (GEN ? A.geo_step : 1)]);
+                det = S::from_pair(gp[D * D * (GEN ? A.geo_step : 1)]);
+            };
+            if (!GEN) load_geo();
             typename S::Acc s;
             for (int q = 0; q < nq; q++) {
+                if (GEN) {
+                    load_geo();
+                    gp += (D * D + 1) * A.geo_step;
+                }
                 typename S::Acc U[D][D];
                 const float2 *dq = A.qd + (size_t)q * nb * D;
 #pragma unroll 2
@@ -1013,9 +727,9 @@ __global__ void __launch_bounds__(128) k_strain_energy(const StrainArgs A)
                 typename S::Acc dens;
                 S::fma(dens, lam, S::mul(tr, tr));
                 S::fma(dens, mu, S::val(sh));
-                S::fma(s, S::from_pair(__ldg(A.qw + q)), S::val(dens));
+                S::fma(s, GEN ? det : S::from_pair(__ldg(A.qw + q)), S::val(dens));
             }
-            const double sd = S::to_double(S::mul(S::val(s), det));
+            const double sd = S::to_double(GEN ? S::val(s) : S::mul(S::val(s), det));
             const double r = A.rho[e];
             A.out[e] = g * simp_dE(A.sp, r) * sd;
             mine += simp_E(A.sp, r) * sd;
@@ -1026,7 +740,7 @@ __global__ void __launch_bounds__(128) k_strain_energy(const StrainArgs A)
 
 // The strain energy density at quadrature point q of a cell whose
 // displacements are staged at us[(b d + i) * ustride] (reference gradients at
-// the point dq[b][m], G row-major), times the point's weight.
+// the point dq[b][m], G row-major).
 template <int D, bool PAIR>
 __device__ __forceinline__ typename SArith<PAIR>::V
 point_energy(const StrainArgs &A, const typename SArith<PAIR>::V *us, int ustride, int q,
@@ -1073,7 +787,7 @@ point_energy(const StrainArgs &A, const typename SArith<PAIR>::V *us, int ustrid
     typename S::Acc dens;
     S::fma(dens, lam, S::mul(tr, tr));
     S::fma(dens, mu, S::val(sh));
-    return S::mul(S::from_pair(__ldg(A.qw + q)), S::val(dens));
+    return S::val(dens);
 }
 
 // The same sensitivities with a warp per cell, for cells with many nodes and
@@ -1105,13 +819,22 @@ __global__ void __launch_bounds__(128) k_strain_energy_warp(const StrainArgs A)
         const float2 *gp = A.geo + e * A.geo_stride;
 #pragma unroll
         for (int t = 0; t < D * D; t++) G[t] = S::from_pair(gp[t]);
-        const V det = S::from_pair(gp[D * D]);
+        V det = S::from_pair(gp[D * D]);
         V sv = S::from_pair(make_float2(0.f, 0.f));
-        for (int q = lane; q < A.nq; q += 32) sv = S::sum(sv, point_energy<D, PAIR>(A, us, 1, q, G, lam, mu));
+        for (int q = lane; q < A.nq; q += 32) {
+            if (A.general) {
+                const float2 *gq = gp + q * (D * D + 1);
+#pragma unroll
+                for (int t = 0; t < D * D; t++) G[t] = S::from_pair(gq[t]);
+                det = S::from_pair(gq[D * D]);
+            }
+            const V en = point_energy<D, PAIR>(A, us, 1, q, G, lam, mu);
+            sv = S::sum(sv, S::mul(A.general ? det : S::from_pair(__ldg(A.qw + q)), en));
+        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sv = S::sum(sv, S::shfl_xor(sv, o));
         if (lane == 0) {
-            const double sd = S::to_double(S::mul(sv, det));
+            const double sd = S::to_double(A.general ? sv : S::mul(sv, det));
             const double r = A.rho[e];
             A.out[e] = g * simp_dE(A.sp, r) * sd;
             mine += simp_E(A.sp, r) * sd;
@@ -1227,7 +950,7 @@ __global__ void __launch_bounds__(128) k_strain_hex_sf(const StrainArgs A, const
         const float2 *gp = A.geo + e * A.geo_stride;
 #pragma unroll
         for (int t = 0; t < D * D; t++) G[t] = S::from_pair(gp[t]);
-        const V det = S::from_pair(gp[D * D]);
+        V det = S::from_pair(gp[D * D]);
         // third index at each point q1 + n q2 + n2 q3, and the density there
         V sv = S::from_pair(make_float2(0.f, 0.f));
         for (int p = lane; p < n3; p += 32) {
@@ -1247,13 +970,19 @@ __global__ void __launch_bounds__(128) k_strain_hex_sf(const StrainArgs A, const
                 Uv[i][1] = S::val(d2);
                 Uv[i][2] = S::val(d3);
             }
-            const V w = S::mul(S::mul(s_w[q1], s_w[q2]), s_w[q3]);
+            if (A.general) {
+                const float2 *gq = gp + p * (D * D + 1);
+#pragma unroll
+                for (int t = 0; t < D * D; t++) G[t] = S::from_pair(gq[t]);
+                det = S::from_pair(gq[D * D]);
+            }
+            const V w = A.general ? det : S::mul(S::mul(s_w[q1], s_w[q2]), s_w[q3]);
             sv = S::sum(sv, S::mul(w, density_from_grad<D, PAIR>(Uv, G, lam, mu)));
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sv = S::sum(sv, S::shfl_xor(sv, o));
         if (lane == 0) {
-            const double sd = S::to_double(S::mul(sv, det));
+            const double sd = S::to_double(A.general ? sv : S::mul(sv, det));
             const double r = A.rho[e];
             A.out[e] = g * simp_dE(A.sp, r) * sd;
             mine += simp_E(A.sp, r) * sd;
@@ -1261,6 +990,135 @@ __global__ void __launch_bounds__(128) k_strain_hex_sf(const StrainArgs A, const
     }
     if (A.c) grid_sum_last_block(mine, A.partial, A.counter, A.c);
 }
+
+// General trilinear hexahedra of order 1 (float pairs), one thread per cell.  The
+// eight Gauss points are the corners of a cube, so the reference displacement
+// gradient at all of them is a Walsh transform each way: with the differences (bit
+// set) and sums (bit clear) of the corner values along the axes, w_b, and a =
+// 1 / sqrt(3), the derivative along axis 1 at the signs (s2, s3) is
+//     (w_100 + s2 a w_110 + s3 a w_101 + s2 s3 a^2 w_111) / 4
+// (and so on), about 150 float-pair sums in place of 576 multiply-adds; the 1 / 16
+// of the energy is applied at the end.  u is read from the cell's nodes, the
+// geometry of the points (80 bytes each) in planes over the cells: 123 MB for
+// 192,000 cells, which bounds the kernel.  (In the gather over the cached element
+// matrices, fused with the assembly, the sensitivities took 340 us on the jittered
+// 120x40x40 hexahedra.)
+__global__ void __launch_bounds__(128, 5) k_strain_hex8(const StrainArgs A)
+{
+    using S = SArith<true>;
+    // derivative along axis m of component i at the signs s of the other two axes (the
+    // lower axis in bit 0), times 4, at us[((3 m + i) 4 + s) 128 + thread]: in registers,
+    // with the eight points unrolled, the kernel waited on instruction fetches (80 us)
+    __shared__ float2 us[36 * 128];
+    const int tid = threadIdx.x;
+    const double g = A.gscale ? *A.gscale : -1.0;
+    const df lam = S::from_pair(A.lam), mu = S::from_pair(A.mu);
+    const df a1 = df_from_double(0.57735026918962576451), a2 = df_from_double(1.0 / 3.0);
+    double mine = 0.0;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + tid; e < A.nc; e += (int64_t)gridDim.x * blockDim.x) {
+        int32_t nd[8];
+#pragma unroll
+        for (int b = 0; b < 8; b++) nd[b] = __ldg(A.cell_node + e * 8 + b);
+#pragma unroll 1
+        for (int i = 0; i < 3; i++) {
+            df w[8];
+#pragma unroll
+            for (int b = 0; b < 8; b++) w[b] = S::from_u(__ldg(A.u + 3 * (int64_t)nd[b] + i));
+#pragma unroll
+            for (int m = 0; m < 3; m++)
+#pragma unroll
+                for (int b = 0; b < 8; b++)
+                    if (!(b & (1 << m))) {
+                        const df lo = w[b], hi = w[b | (1 << m)];
+                        w[b] = df_add_lazy(lo, hi);
+                        w[b | (1 << m)] = df_add_lazy(hi, df_neg(lo));
+                    }
+            w[3] = df_mul(w[3], a1);
+            w[5] = df_mul(w[5], a1);
+            w[6] = df_mul(w[6], a1);
+            w[7] = df_mul(w[7], a2);
+#pragma unroll
+            for (int m = 0; m < 3; m++) {
+                const int p = m == 0 ? 1 : 0, r = m == 2 ? 1 : 2;   // the other axes
+                const df c0 = w[1 << m], cp = w[1 << m | 1 << p], cr = w[1 << m | 1 << r], cc = w[7];
+                const df pl = df_add_lazy(c0, df_neg(cp)), ph = df_add_lazy(c0, cp);
+                const df ql = df_add_lazy(cr, df_neg(cc)), qh = df_add_lazy(cr, cc);
+                float2 *o = us + (3 * m + i) * 4 * 128 + tid;
+                const df v[4] = {df_add_lazy(pl, df_neg(ql)), df_add_lazy(ph, df_neg(qh)), df_add_lazy(pl, ql),
+                                 df_add_lazy(ph, qh)};
+#pragma unroll
+                for (int k = 0; k < 4; k++) o[k * 128] = make_float2(v[k].h, v[k].l);
+            }
+        }
+        S::Acc s;
+        const float2 *gp = A.geo + e;
+#pragma unroll 1
+        for (int q = 0; q < 8; q++, gp += 10 * A.geo_step) {
+            df G[9], Uv[3][3];
+#pragma unroll
+            for (int t = 0; t < 9; t++) G[t] = S::from_pair(__ldcs(gp + t * A.geo_step));
+            const df wd = S::from_pair(__ldcs(gp + 9 * A.geo_step));
+            const int k[3] = {q >> 1, (q & 1) | ((q >> 2) << 1), q & 3};
+#pragma unroll
+            for (int i = 0; i < 3; i++)
+#pragma unroll
+                for (int m = 0; m < 3; m++) Uv[i][m] = S::from_pair(us[((3 * m + i) * 4 + k[m]) * 128 + tid]);
+            S::fma(s, wd, density_from_grad<3, true>(Uv, G, lam, mu));
+        }
+        const double sd = 0.0625 * S::to_double(S::val(s));
+        const double r = A.rho[e];
+        A.out[e] = g * simp_dE(A.sp, r) * sd;
+        mine += simp_E(A.sp, r) * sd;
+    }
+    if (A.c) grid_sum_last_block(mine, A.partial, A.counter, A.c);
+}
+
+// At mesh creation: G = J^-1 and w |det J| of general cells at the Gauss points, in
+// FP64, stored as float pairs.
+template <int D>
+__global__ void k_point_geometry(int64_t nc, int nq, const double *__restrict__ xcell, const double *__restrict__ qw,
+                                 const double *__restrict__ dgeo, int64_t stride, int64_t step, float2 *__restrict__ geo)
+{
+    constexpr int NV = 1 << D;
+    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nc * nq; x += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t e = x / nq;
+        const int q = (int)(x - e * nq);
+        const double *xv = xcell + e * NV * D;
+        double J[D][D] = {};   // from the edge vectors: the rounding does not grow with the cell's distance from the origin
+        for (int v = 1; v < NV; v++)
+            for (int i = 0; i < D; i++)
+                for (int m = 0; m < D; m++) J[i][m] += (xv[v * D + i] - xv[i]) * dgeo[(q * NV + v) * D + m];
+        double G[D * D], det;
+        if constexpr (D == 2) {
+            det = J[0][0] * J[1][1] - J[0][1] * J[1][0];
+            G[0] = J[1][1] / det;
+            G[1] = -J[0][1] / det;
+            G[2] = -J[1][0] / det;
+            G[3] = J[0][0] / det;
+        } else {
+            double C[3][3];   // cofactors
+            for (int i = 0; i < 3; i++)
+                for (int m = 0; m < 3; m++) {
+                    const int i1 = (i + 1) % 3, i2 = (i + 2) % 3, m1 = (m + 1) % 3, m2 = (m + 2) % 3;
+                    C[i][m] = J[i1][m1] * J[i2][m2] - J[i1][m2] * J[i2][m1];
+                }
+            det = J[0][0] * C[0][0] + J[0][1] * C[0][1] + J[0][2] * C[0][2];
+            for (int i = 0; i < 3; i++)
+                for (int m = 0; m < 3; m++) G[m * 3 + i] = C[i][m] / det;
+        }
+        float2 *o = geo + e * stride + (int64_t)q * (D * D + 1) * step;
+        auto put = [&](int t, double v) {
+            const float h = __double2float_rn(v);
+            o[t * step] = make_float2(h, __double2float_rn(v - (double)h));
+        };
+        for (int t = 0; t < D * D; t++) put(t, G[t]);
+        put(D * D, qw[q] * fabs(det));
+    }
+}
+
+// One thread per cell reads the geometry of general cells in planes over the cells,
+// a warp per cell point after point.
+bool point_planes(const soptx_mesh_s &m) { return !m.d.ssf && (int64_t)m.h.nb * m.d.snq < 256; }
 
 template <int D, bool CACHED, bool UNIF>
 cudaError_t pairs_launch(const soptx_mesh_s &m, const double *rho, double *vals, cudaStream_t st)
@@ -1303,63 +1161,11 @@ cudaError_t pairs_launch(const soptx_mesh_s &m, const double *rho, double *vals,
     return cudaGetLastError();
 }
 
-template <int D, int NB, int MINB>
-cudaError_t rows_launch(const soptx_mesh_s &m, const double *rho, double *vals, cudaStream_t st)
-{
-    const auto &h = m.h;
-    ContractArgs A;
-    A.nn = h.nn;
-    A.max_deg = h.max_deg;
-    A.nrec = m.d.cnrec;
-    A.ticket = m.d.cticket;
-    A.inc_e = m.d.cinc_e;
-    A.inc_a = m.d.cinc_a;
-    A.rec = m.d.crec;
-    A.cgeo = m.d.cgeo;
-    A.Mf = m.d.Mf;
-    A.Edf = m.d.Edf;
-    A.rho = rho;
-    A.sp = simp_params(m.mat);
-    A.lam = (float)m.mat.lam;
-    A.mu = (float)m.mat.mu;
-    A.vals = vals;
-    constexpr int NPW = 32 / NB;
-    const size_t mbytes = (size_t)NB * NB * MPad<D>::n * sizeof(float);
-    const size_t per_warp = (size_t)NPW * D * D * h.max_deg * sizeof(float2);
-    // MINB CTAs must fit in the SM's 228 KiB of shared memory (1 KiB of it reserved per CTA)
-    const size_t cta_smem = std::min<size_t>(200 * 1024, (228 * 1024) / MINB - 1024);
-    if (cta_smem < mbytes + per_warp) return cudaErrorInvalidConfiguration;
-    const int wpb = (int)std::max<size_t>(1, std::min<size_t>(8, (cta_smem - mbytes) / per_warp));
-    const size_t smem = mbytes + per_warp * wpb;
-    auto kern = k_contract_rows<D, NB, MINB>;
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
-    // persistent: the CTAs that fit at once, each warp taking many rounds
-    int dev = 0, sms = 0, per_sm = 0;
-    err = cudaGetDevice(&dev);
-    if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (err == cudaSuccess) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, wpb * 32, smem);
-    if (err != cudaSuccess) return err;
-    const int64_t groups = (h.nn + NPW - 1) / NPW;
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((groups + wpb - 1) / wpb, (int64_t)sms * std::max(per_sm, 1)));
-    // (as a dependent launch of the moduli kernel the separate call was 3% faster,
-    // but in the one-call step its CTAs took the SMs the strain-energy kernel
-    // beside it had been getting: slower steps)
-    kern<<<grid, wpb * 32, smem, st>>>(A);
-    return cudaGetLastError();
-}
-
-
 }  // namespace
 
-// CTAs per SM each node-owner layout (3D) is compiled for (its register cap).
-static int rows_minb(int nb) { return nb >= 20 ? 1 : 2; }
-
-// Whether the contraction serves this cell type.  2D (the pair kernel): the
-// reference integrals fit in shared memory and a node's block row, twice its
-// degree, fits the tables' 11 bits.  3D (the node-owner kernel): a compiled
-// layout, and the reference integrals plus one warp's row accumulators (at the
-// largest node degree) fit in a CTA's share of shared memory.
+// Whether the pair kernel serves this 2D cell type: the reference integrals fit in
+// shared memory and a node's block row, twice its degree, fits the tables' 11
+// bits.  3D: the limits of the node-owner schedule (soptx_host_row_tables, host only).
 bool contract_fits(int dim, int nb, int max_deg)
 {
     if (dim == 2) return nb <= 16 && 2 * max_deg <= 2047;
@@ -1367,7 +1173,7 @@ bool contract_fits(int dim, int nb, int max_deg)
     if (dim != 3 || !(nb == 4 || nb == 8 || nb == 10 || nb == 20 || nb == 27) || max_deg > 512) return false;
     const size_t mbytes = (size_t)nb * nb * 12 * sizeof(float);
     const size_t per_warp = (size_t)(32 / nb) * 9 * max_deg * sizeof(float2);
-    const size_t cta_smem = std::min<size_t>(200 * 1024, (228 * 1024) / rows_minb(nb) - 1024);
+    const size_t cta_smem = std::min<size_t>(200 * 1024, (228 * 1024) / (nb >= 20 ? 1 : 2) - 1024);
     return mbytes + per_warp <= cta_smem;
 }
 
@@ -1400,29 +1206,29 @@ bool pairs_fit(int dim, int nb, int max_deg)
     return (dim == 2 || dim == 3) && nb <= 255 && (int64_t)dim * max_deg <= 2047;
 }
 
-// Element moduli as float pairs (k_prep of the gather), then the contraction (or,
-// for the cached FP64 element matrices of 2D meshes, the pair kernel reading them).
+// Element moduli as float pairs (k_prep of the gather), then the pair kernel: over
+// the one matrix of a uniform mesh, the cached FP64 element matrices or the contraction.
 cudaError_t launch_contract_assemble(const soptx_mesh_s &m, const double *rho, double *vals, cudaStream_t st)
 {
-    const auto &h = m.h;
     cudaError_t err = launch_prep(m, rho, nullptr, st);
-    if (err != cudaSuccess) return err;
-    if (m.d.puniform) {
-        if (m.d.ptiles == 0) return cudaSuccess;
-        return h.dim == 3 ? pairs_launch<3, false, true>(m, rho, vals, st)
-                          : pairs_launch<2, false, true>(m, rho, vals, st);
-    }
-    if (h.dim == 2) {
-        if (m.d.ptiles == 0) return cudaSuccess;
-        return m.d.pcached ? pairs_launch<2, true, false>(m, rho, vals, st)
-                           : pairs_launch<2, false, false>(m, rho, vals, st);
-    }
-    if (h.nn == 0 || h.nnz == 0) return cudaSuccess;
-#define SOPTX_CT(NBB, MINB)                                     \
-    if (h.nb == NBB) return rows_launch<3, NBB, MINB>(m, rho, vals, st);
-    SOPTX_CT(4, 2) SOPTX_CT(8, 2) SOPTX_CT(10, 2) SOPTX_CT(20, 1) SOPTX_CT(27, 1)
-#undef SOPTX_CT
-    return cudaErrorInvalidValue;
+    if (err != cudaSuccess || m.d.ptiles == 0) return err;
+    return m.d.puniform  ? pairs_launch<2, false, true>(m, rho, vals, st)
+           : m.d.pcached ? pairs_launch<2, true, false>(m, rho, vals, st)
+                         : pairs_launch<2, false, false>(m, rho, vals, st);
+}
+
+cudaError_t launch_point_geometry(const soptx_mesh_s &m, cudaStream_t st)
+{
+    const auto &h = m.h;
+    const int ng = h.dim * h.dim + 1;
+    const bool pl = point_planes(m);
+    const int64_t stride = pl ? 1 : (int64_t)m.d.snq * ng, step = pl ? h.nc : 1;
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((h.nc * m.d.snq + 255) / 256, 152 * 16));
+    if (h.dim == 2)
+        k_point_geometry<2><<<grid, 256, 0, st>>>(h.nc, m.d.snq, m.d.xcell, m.d.qw, m.d.qdgeo, stride, step, m.d.sgeo);
+    else
+        k_point_geometry<3><<<grid, 256, 0, st>>>(h.nc, m.d.snq, m.d.xcell, m.d.qw, m.d.qdgeo, stride, step, m.d.sgeo);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_strain_sensitivity(const soptx_mesh_s &m, const double *rho, const double *u, double *out,
@@ -1440,6 +1246,13 @@ cudaError_t launch_strain_sensitivity(const soptx_mesh_s &m, const double *rho, 
     A.sp = simp_params(m.mat);
     A.geo = m.d.sgeo;
     A.geo_stride = m.path == SOPTX_PATH_UNIFORM ? 0 : h.dim * h.dim + 1;
+    A.general = h.nonaffine;
+    A.geo_step = 1;
+    if (A.general) {
+        const bool pl = point_planes(m);
+        A.geo_stride = pl ? 1 : (int64_t)m.d.snq * (h.dim * h.dim + 1);
+        A.geo_step = pl ? h.nc : 1;
+    }
     A.qw = m.d.sq;
     A.qd = m.d.sq + m.d.snq;
     auto pair = [](double x) {
@@ -1479,6 +1292,12 @@ cudaError_t launch_strain_sensitivity(const soptx_mesh_s &m, const double *rho, 
         k<<<(int)grid, 128, smem, st>>>(A);
         return cudaGetLastError();
     }
+    if (A.general && h.dim == 3) {   // order 1
+        int64_t grid = std::max<int64_t>(1, std::min<int64_t>((h.nc + 127) / 128, m.d.scratch_len));
+        if (max_grid > 0) grid = std::min<int64_t>(grid, max_grid);
+        k_strain_hex8<<<(int)grid, 128, 0, st>>>(A);
+        return cudaGetLastError();
+    }
     // threads per block: a power of two whose staging fits in 96 KiB
     int T = 128;
     while (T > 32 && (size_t)T * h.nb * h.dim * vb > 96 * 1024) T >>= 1;
@@ -1486,6 +1305,8 @@ cudaError_t launch_strain_sensitivity(const soptx_mesh_s &m, const double *rho, 
     int64_t grid = std::max<int64_t>(1, std::min<int64_t>((h.nc + T - 1) / T, m.d.scratch_len));
     if (max_grid > 0) grid = std::min<int64_t>(grid, max_grid);
     void (*k)(StrainArgs) = nullptr;
+    if (A.general)   // bilinear quadrilaterals of order 1 and 2 (FP64 element matrices)
+        k = h.nb == 4 ? k_strain_energy<2, true, 4, true> : k_strain_energy<2, true, 9, true>;
 #define SOPTX_SE(DD, NBB)                                                                                     \
     if (h.dim == DD && (NBB == 0 || h.nb == NBB) && !k)                                                      \
         k = f32 ? k_strain_energy<DD, false, NBB> : k_strain_energy<DD, true, NBB>;

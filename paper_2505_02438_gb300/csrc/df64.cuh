@@ -175,6 +175,17 @@ __device__ __forceinline__ double pair_to_double(float s, float c)
     return __dadd_rn(f32_to_f64_bits(s), f32_to_f64_bits(c));
 }
 
+// The same in 13 instructions: the halves are widened by a sign-extending shift
+// and an exponent rebias without a test for zero or denormal floats, which turn
+// into values below 2^-126; only s = c = 0 is set to zero again.
+__device__ __forceinline__ double pair_to_double_rebias(float s, float c)
+{
+    const int a = __float_as_int(s), b = __float_as_int(c);
+    const double r = __dadd_rn(__hiloint2double(((a >> 3) & (int)0x8fffffff) + 0x38000000, a << 29),
+                               __hiloint2double(((b >> 3) & (int)0x8fffffff) + 0x38000000, b << 29));
+    return s == 0.f && c == 0.f ? 0.0 : r;
+}
+
 // Sum without the final renormalisation (s, e): enough when the result only
 // feeds further pair arithmetic.
 __device__ __forceinline__ df df_add_lazy(df a, df b)

@@ -89,6 +89,29 @@ bool setup_host_mesh(int dim, int cell, int order, int64_t nv, const double *coo
                      const int32_t *cv, const RefElement &ref, HostMesh &hm, std::string &err);
 void build_csr(const HostMesh &hm, std::vector<int64_t> &indptr, std::vector<int32_t> &indices);
 
+// ---------------------------------------------------------------- block rows
+// Tables of the block-row kernel of 3D meshes (blockrows.cu, where the layout is described).
+constexpr int kBlockHead = 5;   // words before a record's nodes
+struct BlockLimits {
+    int blocks = 432;    // row blocks of a chunk (a larger node is a chunk of its own)
+    int cells = 110;     // cells of a chunk
+    int nodes = 192;     // nodes of a chunk
+    bool sym = true;        // one lane for both blocks of a pair inside a chunk (K_e^0 symmetric to the last bit wanted)
+    bool by_code = false;   // pairs with the same number of cells in the order of their first local pair
+    int cap = 6;         // cells per lane before a pair is shared by several lanes
+};
+struct BlockTables {
+    std::vector<uint32_t> blob;   // the chunks' records, each a whole number of 16-byte units
+    std::vector<uint32_t> coff;   // [nchunks + 1] their starts in 16-byte units
+    int64_t nchunks = 0, rows = 0;
+    int cell_bits = 0;            // bits of a record that name the chunk's cell
+    int max_rows = 0;             // most record rows of a chunk
+    int max_blob = 0;             // largest record in 16-byte units
+    int max_cells = 0, max_stage = 0, max_nodes = 0;   // most cells, staged values and nodes of a chunk
+};
+bool build_block_tables(const HostMesh &hm, const double *coords, const int32_t *cv, const BlockLimits &lim,
+                        BlockTables &T);
+
 // ---------------------------------------------------------------- device mesh
 struct DeviceMesh {
     int64_t *indptr = nullptr;     // [ndof+1]
@@ -120,37 +143,41 @@ struct DeviceMesh {
     // general path
     float2 *udf = nullptr;         // [ndof] u as float pairs (general path; lattice: one-call step)
     double *part = nullptr;        // [nc][nb] per-(cell, node) partials of u_e^T K_e^0 u_e
-    // meshes of affine cells: strain-energy sensitivities (contract.cu)
+    // meshes of affine cells, general cells with FP64 element matrices: strain-energy
+    // sensitivities (contract.cu)
     bool strain = false;           // the sensitivities take k_strain_energy
-    float2 *sgeo = nullptr;        //   [nc, or 1 when uniform][d*d + 1] G and |det J| as float pairs
+    float2 *sgeo = nullptr;        //   [nc, or 1 when uniform][d*d + 1] G and |det J| as float pairs;
+                                   //   general cells: G and w |det J| at every point (StrainArgs)
     float2 *sq = nullptr;          //   quadrature: weights [snq], reference gradients [snq][nb][d]
     int snq = 0;
     float2 *ssf = nullptr;         //   hexahedra of order 2, 3: 1D weights, basis values and derivatives,
                                    //   local nodes' lattice indices (k_strain_hex_sf)
-    // FP32 element matrices of affine cells: assembled by contraction per call
-    bool contract = false;         // the assembly takes k_contract_pairs (2D) or k_contract_rows (3D)
-    float4 *cgeo = nullptr;        //   [nc][2 or 3] G and |det J| in FP32
-    float *Mf = nullptr;           //   [nb][nb][4 or 12] reference integrals in FP32
-    // node pairs in tiles of 32 (2D: {a, b} with b = a or b after a; 3D: every
-    // ordered pair); also for the cached FP64 element matrices of 2D affine meshes
-    // (pcached) and the one element matrix of a uniform mesh (puniform)
-    bool pcached = false;
-    bool puniform = false;         //   the pair kernel over the one element matrix of a uniform mesh
+    // 2D meshes: node pairs in tiles of 32 (contract.cu)
+    bool contract = false;         // FP32 element matrices of affine cells, contracted per call
+    bool pcached = false;          //   cached FP64 element matrices of affine cells
+    bool puniform = false;         //   the one element matrix of a uniform mesh
+    float4 *cgeo = nullptr;        //   [nc][2] G and |det J| in FP32
+    float *Mf = nullptr;           //   [nb][nb][4] reference integrals in FP32
     int64_t ptiles = 0;            //   tiles
     uint32_t *ptoff = nullptr;     //   [8 chunks + 16] first record of each tile / 32
     uint32_t *pia = nullptr;       //   [256 chunks] value index of block (a, b) / d
-    uint32_t *pib = nullptr;       //   [256 chunks] value index of block (b, a) / d (3D: = pia)
+    uint32_t *pib = nullptr;       //   [256 chunks] value index of block (b, a) / d
     uint32_t *pmeta = nullptr;     //   [256 chunks] cells | a's row length << 10 | b's << 21
     int32_t *pre = nullptr;        //   per record: the cell (ascending per pair)
     uint16_t *prm = nullptr;       //   per record: a_loc nb + b_loc (pcached, puniform: a_loc << 8 | b_loc)
     float4 *pblk = nullptr;        //   pcached: per record its 2 x 2 block of K_e^0 (2 float4s)
-    // 3D: each node's cells as a chain, walked by the node's group of lanes
-    int4 *cnrec = nullptr;         //   [nn] nodes by incident-cell count, largest first: row block
-                                   //   offset (2 ints), first incidence, cells << 16 | degree
-    int32_t *cinc_e = nullptr;     //   [ninc] each node's cells in the contraction's chain order
-    uint8_t *cinc_a = nullptr;     //   [ninc] the node's local index in those cells
-    uint16_t *crec = nullptr;      //   [ninc][nb] per lane: block p, local node b << 9, first/last flags
-    unsigned *cticket = nullptr;   //   [2] work counter and finished warps or CTAs (zero between calls)
+    // 3D meshes: chunks of complete rows (blockrows.cu)
+    int64_t bchunks = -1;          //   chunks (-1: the mesh's assembly is another kernel's)
+    int bsmem = 0;                 //   shared memory of a CTA
+    int bsrc = 0;                  //   where the blocks come from (kBlockContract, ...)
+    int bmax_blob = 0, bmax_cells = 0, bmax_stage = 0, bmax_rows = 0, bcell_bits = 0;   // see BlockTables
+    uint4 *bblob = nullptr;        //   chunk records
+    uint32_t *bcoff = nullptr;     //   [bchunks + 1] their starts
+    float4 *bcell = nullptr;       //   kBlockContract: [nc][3] G, |det J| in FP32
+    float *bM = nullptr;           //   kBlockContract: reference integrals [nb][nb][12] in FP32
+    float4 *bkblk = nullptr;       //   kBlockUniform: the blocks of the one element matrix
+                                   //   kBlockStream: every record's block, in the kernel's order
+    unsigned *cticket = nullptr;   // [4] chunk counter, finished CTAs (both zero between calls), error flag
     // equilibrium solve (allocated by the first soptx_solve_cg)
     double *cg = nullptr;          // r z p q diag [ndof], scalars, partials, counters
     cudaGraphExec_t cg_exec = nullptr; // the CG iterations between two checks, as a graph
@@ -213,11 +240,18 @@ cudaError_t launch_gather(const soptx_mesh_s &m, const double *rho, const double
                           double *c, const double *gscale, cudaStream_t st);
 int gather_finalize_grid(int64_t nc);
 cudaError_t launch_prep(const soptx_mesh_s &m, const double *rho, const double *u, cudaStream_t st);
+// blockrows.cu
+enum { kBlockContract = 0, kBlockUniform = 1, kBlockStream = 2 };
+int64_t block_row_bytes();   // a record row of streamed blocks
+int64_t block_smem(int src, int nb, const BlockTables &T);
+cudaError_t launch_block_stream(const soptx_mesh_s &m, cudaStream_t st);
+cudaError_t launch_block_rows(const soptx_mesh_s &m, const double *rho, double *vals, cudaStream_t st);
 // contract.cu
 bool contract_fits(int dim, int nb, int max_deg);
 bool pairs_fit(int dim, int nb, int max_deg);
 cudaError_t launch_contract_assemble(const soptx_mesh_s &m, const double *rho, double *vals, cudaStream_t st);
 cudaError_t launch_pair_blocks(const soptx_mesh_s &m, int64_t nrec, cudaStream_t st);
+cudaError_t launch_point_geometry(const soptx_mesh_s &m, cudaStream_t st);
 // max_grid > 0 caps the blocks (the kernel loops over the cells): beside a
 // persistent assembly, a block per SM leaves it the rest of the GPU
 cudaError_t launch_strain_sensitivity(const soptx_mesh_s &m, const double *rho, const double *u, double *out,

@@ -266,6 +266,7 @@ cudaError_t launch_assemble(const soptx_mesh_s &m, const double *rho, double *va
 {
     if (m.h.nn == 0 || m.h.nnz == 0) return cudaSuccess;
     if (m.path == SOPTX_PATH_LATTICE) return launch_lattice_assemble(m, rho, vals, st);
+    if (m.d.bchunks >= 0) return launch_block_rows(m, rho, vals, st);
     if (m.d.contract || m.d.pcached || m.d.puniform) return launch_contract_assemble(m, rho, vals, st);
     return launch_gather(m, rho, nullptr, vals, nullptr, nullptr, nullptr, st);
 }
@@ -289,20 +290,21 @@ cudaError_t launch_step(const soptx_mesh_s &m, const double *rho, const double *
     if (m.path == SOPTX_PATH_LATTICE && m.d.sectors && m.h.nc > 0)
         return launch_lattice_step(m, rho, u, vals, dc, c, st, gscale);
     if (m.d.strain && m.d.side && m.h.nc > 0 && m.h.nnz > 0 &&
-        (((m.d.contract || m.d.pcached) && m.h.dim == 2) || m.d.puniform)) {
-        // the 2D pair kernel fills every SM with a persistent grid that takes
-        // its work from a counter: the sensitivities go first, on the mesh's second
-        // stream (highest priority) with one block per SM, and the contraction's
-        // CTAs take the rest of the GPU and, as those blocks finish, their slots
-        // (in 3D, with one block of 64 threads per SM beside the node-owner
-        // contraction, the sensitivities outlasted it: P2 tets 304.5 -> 345.8 us)
+        (m.d.bchunks >= 0 || m.d.contract || m.d.pcached || m.d.puniform)) {
+        // the pair and block-row kernels fill every SM with a persistent grid that
+        // takes its work from a counter: the sensitivities go first, on the mesh's
+        // second stream (highest priority) with a few blocks per SM, and the assembly's
+        // CTAs take the rest of the GPU and, as those blocks finish, their slots.
+        // Blocks per SM, step us: P3 triangles 400x200 FP64 281 at one, 239 at four
+        // (the float-pair sensitivity outlasted the assembly at one), FP32 172 / 176;
+        // P2 tets 60x20x20 FP64 364 / 340, FP32 233 / 224
         int dev = 0, sms = 0;
         cudaError_t err = cudaGetDevice(&dev);
         if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (err == cudaSuccess) err = cudaEventRecord(m.d.ev[0], st);
         if (err == cudaSuccess) err = cudaStreamWaitEvent(m.d.side, m.d.ev[0], 0);
         if (err == cudaSuccess)
-            err = launch_strain_sensitivity(m, rho, u, dc, c, gscale, m.d.side, sms);
+            err = launch_strain_sensitivity(m, rho, u, dc, c, gscale, m.d.side, m.d.contract ? sms : 4 * sms);
         if (err == cudaSuccess) err = cudaEventRecord(m.d.ev[1], m.d.side);
         if (err == cudaSuccess) err = launch_assemble(m, rho, vals, st);
         if (err == cudaSuccess) err = cudaStreamWaitEvent(st, m.d.ev[1], 0);
@@ -321,7 +323,7 @@ cudaError_t launch_step(const soptx_mesh_s &m, const double *rho, const double *
         if (err == cudaSuccess) err = cudaStreamWaitEvent(st, m.d.ev[1], 0);
         return err;
     }
-    if (m.path == SOPTX_PATH_LATTICE || m.h.nc == 0 || m.d.strain) {
+    if (m.path == SOPTX_PATH_LATTICE || m.h.nc == 0 || m.d.strain || m.d.bchunks >= 0) {
         cudaError_t err = launch_assemble(m, rho, vals, st);
         if (err != cudaSuccess) return err;
         return launch_sensitivity(m, rho, u, dc, c, -1.0, gscale, st);

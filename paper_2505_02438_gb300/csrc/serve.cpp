@@ -78,7 +78,12 @@ int64_t max_cells_at_vertex(const soptx_request &r, int nv)
 // most the previous tile's smallest, so a window pads at most 32 times its
 // largest count (at most the most cells at a vertex, c) above its own records,
 // and windows hold 4096 pairs or more but the last.  In 2D with FP64 element
-// matrices each record also carries its 2 x 2 block (32 bytes).
+// matrices each record also carries its 2 x 2 block (32 bytes).  3D meshes hold the
+// block-row kernel's chunk records instead: a chunk ends when its next node would
+// take it past 432 blocks, 110 cells or 192 nodes, so two neighbouring chunks pass one
+// of these together; each (pair, cell) has one lane of a record row (2 bytes, and with
+// FP64 element matrices its streamed block of 72), a pair's shares at most double it, and a
+// chunk's tiles pad 192 lanes by its most rows; 8 bytes per lane of a tile.
 int64_t mesh_bytes_bound(const soptx_request &r)
 {
     static const int nb_tab[4][4] = {{0, 3, 6, 10}, {0, 4, 10, 20}, {0, 4, 9, 16}, {0, 8, 27, 64}};
@@ -90,13 +95,21 @@ int64_t mesh_bytes_bound(const soptx_request &r)
     const int64_t base = ee * 8 /* K_e (cached) */ + ee * 4 /* indices */ + nc * nb * nb * 2 /* pos */ +
                          nc * nb * (4 + 4 + 4 + 1 + 8) /* cell_node, inc, inc_e, inc_a, partials */ +
                          nn * r.dim * (8 + 8) + nn * 20 + nc * 120 + (1 << 20);
+    // general quadrilaterals and hexahedra: the geometry of every Gauss point
+    const int64_t points = nv_tab[r.cell] == (1 << r.dim) && r.cell != SOPTX_TET ? nb * (r.dim * r.dim + 1) * 8 : 0;
     const int64_t c = std::min<int64_t>(max_cells_at_vertex(r, nv_tab[r.cell]), 1023);
-    const int64_t rec = nc * (r.dim == 2 ? nb * (nb + 1) / 2 : nb * nb);
+    if (r.dim == 3) {
+        const int64_t rec = nc * nb * nb, chunks = 2 * (rec / 432 + nc * nb / 110 + nn / 192) + 1;
+        const int64_t lanes = 2 * rec + chunks * 192 * std::max<int64_t>(6, c / 32 + 1);
+        const int64_t per_lane = 2 + 8 + (r.prec == SOPTX_ELEM_FP64 ? 72 : 0);
+        return base + lanes * per_lane + nn * 8 + nc * nb * (4 + 48) + chunks * 64 + nc * points;
+    }
+    const int64_t rec = nc * (nb * (nb + 1) / 2);
     const int64_t windows = rec / 4096 + 1;
     const int64_t padded = rec + windows * 32 * c;
     const int64_t lanes = rec + windows * 32 + 7 * 32;   // and the last chunk of 8 tiles filled
-    const int64_t per_rec = 4 + 2 + (r.dim == 2 && r.prec == SOPTX_ELEM_FP64 ? 32 : 0);
-    return base + padded * per_rec + lanes * 12 + (lanes / 32 + 32) * 4 + 64;
+    const int64_t per_rec = 4 + 2 + (r.prec == SOPTX_ELEM_FP64 ? 32 : 0);
+    return base + nc * points + padded * per_rec + lanes * 12 + (lanes / 32 + 32) * 4 + 64;
 }
 
 }  // namespace
