@@ -1149,8 +1149,9 @@ soptx_status soptx_compliance_vjp(soptx_mesh m, const double *d_rho, const doubl
     cudaStream_t st = (cudaStream_t)stream;
     auto &d = m->d;
     if (d_grad_u && !d.kvals && m->h.nnz > 0) {
-        // K(rho) for 2 g K(rho) u goes into a mesh-owned scratch of 8 nnz bytes, made once;
-        // where that memory cannot be had the product is formed matrix-free instead
+        // the cells' forces, or K(rho) for 2 g K(rho) u, go into a mesh-owned scratch of 8 nnz
+        // bytes, made once; where that memory cannot be had the product is formed
+        // from the element matrices without it
         void *p = nullptr;
         if (dev_alloc(&p, (size_t)m->h.nnz * sizeof(double)) == cudaSuccess) {
             d.kvals = (double *)p;
@@ -1167,6 +1168,9 @@ soptx_status soptx_compliance_vjp(soptx_mesh m, const double *d_rho, const doubl
         return cuda_status(cudaMemsetAsync(d_grad_u, 0, (size_t)m->h.ndof * sizeof(double), st),
                            "soptx_compliance_vjp");
     }
+    if (d_grad_u && d.kvals && vjp_matrix_free(*m))
+        return cuda_status(launch_vjp(*m, d_rho, d_u, d_gout, d_grad_rho, d_grad_u, (float2 *)d.kvals, st),
+                           "soptx_compliance_vjp");
     if (d_grad_u && d.kvals) {
         // one step (K(rho) and the rho-gradient g E' s) then the product with u
         soptx_status s = cuda_status(launch_step(*m, d_rho, d_u, d.kvals, d_grad_rho, nullptr, st, d_gout),

@@ -183,7 +183,8 @@ struct DeviceMesh {
     cudaGraphExec_t cg_exec = nullptr; // the CG iterations between two checks, as a graph
     cudaStream_t cg_cap = nullptr;     // its capture stream
     const void *cg_key[4] = {};        // vals, fixed, u and the iteration count it was made for
-    // K(rho) for the backward's u-gradient (made by the first soptx_compliance_vjp with d_grad_u)
+    // scratch of the backward's u-gradient: the cells' nodal forces or K(rho) (made by the
+    // first soptx_compliance_vjp with d_grad_u)
     double *kvals = nullptr;
     // the step from host buffers (made by the first soptx_step_host)
     double *stage = nullptr;           // rho [nc], u [ndof], dc [nc], c [1] on the device
@@ -219,6 +220,10 @@ cudaError_t launch_sensitivity(const soptx_mesh_s &m, const double *rho, const d
                                double *c, double scale, const double *gscale, cudaStream_t st);
 cudaError_t launch_Ku(const soptx_mesh_s &m, const double *rho, const double *u, const double *gout,
                       double *out, cudaStream_t st);
+// vjp.cu: both gradients of the backward from the cells, without K; f: scratch of nc ldof pairs
+bool vjp_matrix_free(const soptx_mesh_s &m);
+cudaError_t launch_vjp(const soptx_mesh_s &m, const double *rho, const double *u, const double *gout, double *grad_rho,
+                       double *grad_u, float2 *f, cudaStream_t st);
 cudaError_t launch_scaled_product(const soptx_mesh_s &m, const double *vals, const double *u, const double *gout,
                                   double *out, cudaStream_t st);
 int64_t sensitivity_scratch_len(const soptx_mesh_s &m);
