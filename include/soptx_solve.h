@@ -49,9 +49,13 @@ typedef struct {
  *   d_u     : device float64 [ndof]; on entry the prescribed values on the
  *             constrained dofs (and the initial guess elsewhere with
  *             warm_start, else ignored), on exit the solution
- * Runs on `stream` and returns when done: the host reads the residual back
- * every opts->check_every steps.  The first call on a mesh allocates its CG
- * vectors (5 ndof doubles), kept until soptx_mesh_destroy.  Sums are taken in
+ * Runs on `stream` and returns when done; the residual is tested every
+ * opts->check_every steps.  A matrix that fits the SMs' shared memory (up to
+ * about 30 MB) is kept there and the iterations run in one cooperative launch,
+ * which needs all SMs at once; otherwise, or where that launch is refused, in
+ * launches per iteration.  The first call on a mesh allocates its CG vectors (5
+ * ndof doubles) and, for the first form, tables of about 2 bytes per block of
+ * K, kept until soptx_mesh_destroy (without memory for the tables: the second).  Sums are taken in
  * a fixed order, so the iterates are bitwise reproducible.  Calls on one mesh
  * must not overlap.
  * Errors: EINVAL (bad arguments), ENOMEM, ECUDA; a zero diagonal on a free dof

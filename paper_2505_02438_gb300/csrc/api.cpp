@@ -37,7 +37,7 @@ static void free_device(DeviceMesh &d)
                     d.pos, d.geo, d.M, d.K, d.scratch, d.Edf, d.kappa, d.K0, d.sectors, d.udf, d.part,
                     d.inc_e, d.inc_a, d.counter, d.xcell, d.qw, d.qdphi, d.qdgeo, d.cg, d.lat_bad, d.stage,
                     d.kvals, d.sgeo, d.sq, d.ssf, d.cgeo, d.Mf, d.ptoff, d.pia, d.pib, d.pmeta, d.pre, d.prm, d.pblk,
-                    d.bblob, d.bcoff, d.bcell, d.bM, d.bkblk, d.cticket};
+                    d.bblob, d.bcoff, d.bcell, d.bM, d.bkblk, d.cticket, d.rbuf};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (d.cg_exec) cudaGraphExecDestroy(d.cg_exec);

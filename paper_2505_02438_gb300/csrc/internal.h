@@ -183,6 +183,11 @@ struct DeviceMesh {
     cudaGraphExec_t cg_exec = nullptr; // the CG iterations between two checks, as a graph
     cudaStream_t cg_cap = nullptr;     // its capture stream
     const void *cg_key[4] = {};        // vals, fixed, u and the iteration count it was made for
+    // the solve with K in shared memory (cgresident.cu): 0 not looked at yet, 1 in use, -1 not
+    int rstate = 0, rblocks = 0, rsmem = 0;
+    unsigned char *rbuf = nullptr;     // its exchange words and tables
+    unsigned char *rtables = nullptr;  //   first nodes [rblocks + 1]; at the byte offsets below the halo
+    size_t rhoff = 0, rhalo = 0, rlidx = 0;   // starts, the halo nodes and the entries' local nodes
     // scratch of the backward's u-gradient: the cells' nodal forces or K(rho) (made by the
     // first soptx_compliance_vjp with d_grad_u)
     double *kvals = nullptr;
@@ -190,6 +195,12 @@ struct DeviceMesh {
     double *stage = nullptr;           // rho [nc], u [ndof], dc [nc], c [1] on the device
     cudaStream_t side = nullptr;       // second stream: u's copy, the sensitivities, dc and c back
     cudaEvent_t ev[2] = {};            // rho on the device (and all work before it), side stream done
+};
+
+// What the resident solve reports after a launch.
+struct CgResidentOut {
+    int it, converged, error, unused;
+    double rr;   // r.r of the last iterate
 };
 
 struct Material {
@@ -224,6 +235,11 @@ cudaError_t launch_Ku(const soptx_mesh_s &m, const double *rho, const double *u,
 bool vjp_matrix_free(const soptx_mesh_s &m);
 cudaError_t launch_vjp(const soptx_mesh_s &m, const double *rho, const double *u, const double *gout, double *grad_rho,
                        double *grad_u, float2 *f, cudaStream_t st);
+// the solve with K in shared memory (cgresident.cu)
+bool cg_resident_ready(soptx_mesh_s &m, cudaStream_t st);
+cudaError_t cg_resident_run(const soptx_mesh_s &m, const double *vals, const uint8_t *fixed, const double *dinv,
+                            double *u, double *r, double *z, double *p, double *rz, int check_every, int max_iter, double stop,
+                            cudaStream_t st, CgResidentOut *res, bool *launched);
 cudaError_t launch_scaled_product(const soptx_mesh_s &m, const double *vals, const double *u, const double *gout,
                                   double *out, cudaStream_t st);
 int64_t sensitivity_scratch_len(const soptx_mesh_s &m);

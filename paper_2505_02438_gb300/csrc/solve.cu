@@ -1,6 +1,7 @@
 // The step after assembly (include/soptx_solve.h): y = K x on the mesh's CSR
 // values, and Jacobi-preconditioned conjugate gradients for K u = f under
-// Dirichlet constraints.
+// Dirichlet constraints (cgresident.cu has the iterations for matrices that fit the
+// SMs' shared memory).
 //
 //  k_spmv      : four nodes per warp, eight lanes per node; each lane takes
 //                the columns c, c+8, ... of the node's column list (shared by
@@ -476,6 +477,23 @@ soptx_status soptx_solve_cg(soptx_mesh m, const double *d_vals, const uint8_t *d
         res->converged = 1;
         res->rel_residual = r0 == 0.0 ? 0.0 : std::sqrt(rr) / r0;
         return SOPTX_OK;
+    }
+    // K in shared memory and one launch for all iterations, when it fits
+    if (cg_resident_ready(*m, st)) {
+        CgResidentOut out;
+        bool launched = false;
+        e = cg_resident_run(*m, d_vals, d_fixed, diag, d_u, r, z, pv, S + 4, o->check_every, o->max_iter, o->rtol * r0,
+                            st, &out, &launched);
+        if (launched) {
+            if (e != cudaSuccess) return cuda_fail(e, "soptx_solve_cg");
+            if (out.error) SOPTX_FAIL(SOPTX_ECUDA, "soptx_solve_cg: a wait between the blocks ran out");
+            res->iterations = out.it;
+            res->converged = out.converged;
+            res->rel_residual = std::sqrt(out.rr) / r0;
+            return SOPTX_OK;
+        }
+        e = cudaSuccess;
+        cudaGetLastError();   // refused: the loop below
     }
     // One CG iteration: three dependent launches (each is scheduled while the one
     // before it finishes and waits for it before reading anything).
