@@ -141,10 +141,13 @@ __device__ __forceinline__ void grid_sum_last_block_n(double mine, double *__res
     if (!last) return;
     __threadfence();
     double t = 0.0;
-    for (int i = threadIdx.x; i < (int)nblk; i += blockDim.x) t += __ldcg(partial + i);
-    red[threadIdx.x] = t;
+    const int nt = min((int)blockDim.x, 256);   // the threads that sum
+    if ((int)threadIdx.x < nt) {
+        for (int i = threadIdx.x; i < (int)nblk; i += nt) t += __ldcg(partial + i);
+        red[threadIdx.x] = t;
+    }
     __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+    for (int w = nt / 2; w > 0; w >>= 1) {
         if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
         __syncthreads();
     }

@@ -761,6 +761,7 @@ template <int D> struct LatReq {
 };
 constexpr int kGroupMax = 32;
 constexpr int kGroupCtas = 8;   // a portable cluster size
+constexpr int kSingleCtas = 16; // the largest cluster
 template <int D> struct LatGroup {
     int n;
     LatReq<D> r[kGroupMax];
@@ -785,6 +786,31 @@ __global__ void __launch_bounds__(256) k_lattice_step_group(const __grid_constan
     for (int vb = rank; vb < R.sgrid; vb += kGroupCtas)
         lattice_sens_body<D, float2>(R.nx, R.ny, R.nc, R.rho, R.udf, R.sp, R.B, R.gscale, R.dc, R.partial, R.counter,
                                      R.c, vb, R.sgrid, 128);
+}
+
+// One small mesh's step in one launch of two clusters: the first forms the moduli and,
+// after a cluster barrier, K; the second the sensitivities, which need rho and u alone
+// (u's pairs split at every corner, the same pairs).  The same arithmetic in the same
+// order as the three launches of a larger mesh's step.
+template <int D, int WPB>
+__global__ void __launch_bounds__(WPB * 32) k_lattice_step_single(const __grid_constant__ LatReq<D> R)
+{
+    const int rank = (int)(blockIdx.x % kSingleCtas);
+    if (blockIdx.x >= kSingleCtas) {
+        for (int vb = rank; vb < R.sgrid; vb += kSingleCtas)
+            lattice_sens_body<D, double>(R.nx, R.ny, R.nc, R.rho, R.u, R.sp, R.B, R.gscale, R.dc, R.partial, R.counter,
+                                         R.c, vb, R.sgrid, 128);
+        return;
+    }
+    simp_df_body(D, R.nx, R.ny, R.nz, R.nc, R.rho, R.sp, R.Edf, R.node_off, R.K0, R.vals, R.flag, R.gen, R.ndof,
+                 (const double *)nullptr, R.udf, rank, kSingleCtas);
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if constexpr (D == 2)
+        lattice_assemble2_body<WPB, false>(R.nx, R.ny, R.nn, R.chunk, R.node_off, R.Edf, R.kappa, R.vals, R.flag, R.gen,
+                                           R.pbias, R.kscale, rank, kSingleCtas);
+    else
+        lattice_assemble3_body<WPB, false>(R.nx, R.ny, R.nz, R.nn, R.chunk, R.node_off, R.Edf, R.kappa, R.K0, R.rho,
+                                           R.sp, R.vals, R.flag, R.gen, R.pbias, R.kscale, rank, kSingleCtas);
 }
 
 }  // namespace
@@ -940,6 +966,136 @@ cudaError_t launch_lattice_assemble(const soptx_mesh_s &m, const double *rho, do
     return lattice_assemble_u(m, rho, nullptr, vals, st);
 }
 
+// ------------------------------------------------------------- grouped steps
+// Meshes the grouped step serves: 2D and 3D box lattices whose sensitivity
+// splits into Walsh sectors, up to kGroupCells cells in 2D and kGroupCells3 in
+// 3D (a cluster of kGroupCtas CTAs does the whole step; a larger 3D mesh's step
+// takes longer on one cluster than its three launches across the GPU).
+constexpr int64_t kGroupCells = 4096;
+constexpr int64_t kGroupCells3 = 1024;
+// Meshes whose own step is one launch of two clusters.  Three launches and one: calls in
+// a row from C, one call with its synchronisation, calls replayed in a graph, us:
+//   60x20 cells 10.6 18.6  7.0 and  8.2 17.4 6.9;   32x64 11.3 19.5 7.4 and 10.3 19.0 8.0
+//   64x64       10.6 20.0  8.1 and 14.4 23.6 12.8
+//   4x4x4       18.5 27.6 17.0 and 10.3 19.6 8.6;   8x8x8 18.5 28.0 17.3 and 11.1 20.3 9.3
+//   16x8x8      19.7 28.8 17.7 and 16.4 26.0 14.9
+// (from Python 26.8 and 19.6 for all of them: the host).  In 2D the CTAs have 16 warps
+// when 8 would have more than one chunk each: 20x16 8.2 16.3 5.5 with 8 and 8.2 16.9 6.8
+// with 16, 60x20 9.3 18.0 7.5 and 8.2 17.4 6.9.
+constexpr int64_t kSingleCells = 1536;   // in 2D; in 3D kGroupCells3
+constexpr int64_t kSingleWide = 3 * 8 * kSingleCtas;
+static_assert(kSensThreads == 128, "the grouped step replays the 128-thread sensitivity blocks");
+// its 256 threads then sum at most 128 block partials as the 128 of the single step do
+static_assert((kGroupCells + 127) / 128 <= 128, "the grouped step's last-block sum needs <= 128 partials");
+
+bool lattice_groupable(const soptx_mesh_s &m)
+{
+    const auto &h = m.h;
+    return m.path == SOPTX_PATH_LATTICE && (h.dim == 2 || h.dim == 3) && m.d.sectors && m.d.udf && m.d.Edf &&
+           h.nc > 0 && h.nc <= (h.dim == 2 ? kGroupCells : kGroupCells3) &&
+           (int)h.sectors.size() == (h.dim << h.dim) * h.dim;
+}
+
+// The request of one mesh's step, its chunks for `warps` warps.
+template <int D>
+static LatReq<D> group_request(int warps, const soptx_mesh_s &m, const double *rho, const double *u, double *vals,
+                               double *dc, double *c, const double *gscale)
+{
+    const auto &h = m.h;
+    LatReq<D> R;
+    unsigned gen = ++m.lattice_gen;
+    if (gen == 0u) gen = ++m.lattice_gen;
+    R.nx = h.lat_n[0];
+    R.ny = h.lat_n[1];
+    R.nz = D == 3 ? h.lat_n[2] : 1;
+    if (D == 2) {
+        // node chunks of 3 .. 48 for the cluster's warps
+        const int64_t groups = (h.nn + 2) / 3;
+        R.chunk = 3 * (int)std::max<int64_t>(1, std::min<int64_t>(16, groups / warps));
+    } else {
+        // even chunks of at most kChunk nodes, about as many per warp (as in the single step)
+        const int64_t rounds = (h.nn + warps * kChunk - 1) / (warps * kChunk);
+        int chunk = (int)std::max<int64_t>(1, (h.nn + warps * rounds - 1) / (warps * rounds));
+        R.chunk = chunk + (chunk & 1);
+    }
+    R.sgrid = lattice_sens_grid(h.nc);
+    R.gen = gen;
+    R.pbias = 0x38000000u + ((uint32_t)h.lat_kshift << 20);
+    R.nn = h.nn;
+    R.nc = h.nc;
+    R.ndof = h.ndof;
+    R.kscale = std::ldexp(1.0, h.lat_kshift);
+    R.sp = simp_params(m.mat);
+    R.B = sector_table<D>(h.sectors);
+    R.rho = rho;
+    R.u = u;
+    R.gscale = gscale;
+    R.K0 = m.d.K0;
+    R.vals = vals;
+    R.dc = dc;
+    R.c = c;
+    R.partial = m.d.scratch;
+    R.Edf = (float2 *)m.d.Edf;
+    R.udf = m.d.udf;
+    R.node_off = m.d.node_off;
+    R.flag = m.d.lat_bad;
+    R.counter = m.d.counter;
+    R.kappa = (const float2 *)m.d.kappa;
+    return R;
+}
+
+// kern as `clusters` clusters of `ctas` CTAs.
+template <typename P>
+static cudaError_t launch_clusters(void (*kern)(P), int clusters, int ctas, int threads, const P &param, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(clusters * ctas));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = 0;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)ctas;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, param);
+}
+
+template <int D>
+static cudaError_t launch_group_d(const std::vector<int> &ks, const soptx_mesh_s *const *ms, const double *const *rho,
+                                  const double *const *u, double *const *vals, double *const *dc, double *const *c,
+                                  cudaStream_t st)
+{
+    const int n = (int)ks.size();
+    for (int k0 = 0; k0 < n; k0 += kGroupMax) {
+        static thread_local LatGroup<D> G;   // ~24 KB: off the stack
+        G = LatGroup<D>{};
+        G.n = std::min(kGroupMax, n - k0);
+        for (int k = 0; k < G.n; k++) {
+            const int j = ks[k0 + k];
+            G.r[k] = group_request<D>(8 * kGroupCtas, *ms[j], rho[j], u[j], vals[j], dc[j], c[j], nullptr);
+        }
+        cudaError_t err = launch_clusters<const LatGroup<D>>(k_lattice_step_group<D>, G.n, kGroupCtas, 256, G, st);
+        if (err != cudaSuccess) return err;
+    }
+    return cudaSuccess;
+}
+
+// One small mesh's step in one launch.
+template <int D, int WPB>
+static cudaError_t launch_single(const soptx_mesh_s &m, const double *rho, const double *u, double *vals, double *dc,
+                                 double *c, cudaStream_t st, const double *gscale)
+{
+    // (clusters of more than 8 CTAs are launched on request)
+    cudaError_t err = cudaFuncSetAttribute(k_lattice_step_single<D, WPB>,
+                                           cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (err != cudaSuccess) return err;
+    return launch_clusters<const LatReq<D>>(k_lattice_step_single<D, WPB>, 2, kSingleCtas, WPB * 32,
+                                            group_request<D>(WPB * kSingleCtas, m, rho, u, vals, dc, c, gscale), st);
+}
+
 // One call doing both passes: u is split into float pairs once, by the moduli
 // kernel, instead of at every corner of every cell.
 cudaError_t launch_lattice_step(const soptx_mesh_s &m, const double *rho, const double *u, double *vals, double *dc,
@@ -949,6 +1105,13 @@ cudaError_t launch_lattice_step(const soptx_mesh_s &m, const double *rho, const 
         cudaError_t err = lattice_assemble_u(m, rho, nullptr, vals, st);
         if (err != cudaSuccess) return err;
         return launch_lattice_sensitivity(m, rho, u, dc, c, gscale, st);
+    }
+    if (lattice_groupable(m) && m.h.nc <= (m.h.dim == 2 ? kSingleCells : kGroupCells3)) {
+        const cudaError_t err = m.h.dim == 3            ? launch_single<3, 8>(m, rho, u, vals, dc, c, st, gscale)
+                                : m.h.nn > kSingleWide ? launch_single<2, 16>(m, rho, u, vals, dc, c, st, gscale)
+                                                       : launch_single<2, 8>(m, rho, u, vals, dc, c, st, gscale);
+        if (err != cudaErrorLaunchOutOfResources && err != cudaErrorInvalidClusterSize) return err;
+        cudaGetLastError();   // no room for a cluster of 16: the launches below
     }
     if (m.h.dim == 2 && m.d.side) {
         // 2D: the sensitivity runs on the mesh's second stream beside the assembly
@@ -1034,98 +1197,6 @@ void build_lattice_kappa(int dim, const std::vector<double> &K0, int shift, std:
         const float hh = (float)x;
         kappa[t] = make_float2(hh, (float)(x - (double)hh));
     }
-}
-
-// ------------------------------------------------------------- grouped steps
-// Meshes the grouped step serves: 2D and 3D box lattices whose sensitivity
-// splits into Walsh sectors, up to kGroupCells cells in 2D and kGroupCells3 in
-// 3D (a cluster of kGroupCtas CTAs does the whole step; a larger 3D mesh's step
-// takes longer on one cluster than its three launches across the GPU).
-constexpr int64_t kGroupCells = 4096;
-constexpr int64_t kGroupCells3 = 1024;
-static_assert(kSensThreads == 128, "the grouped step replays the 128-thread sensitivity blocks");
-// its 256 threads then sum at most 128 block partials as the 128 of the single step do
-static_assert((kGroupCells + 127) / 128 <= 128, "the grouped step's last-block sum needs <= 128 partials");
-
-bool lattice_groupable(const soptx_mesh_s &m)
-{
-    const auto &h = m.h;
-    return m.path == SOPTX_PATH_LATTICE && (h.dim == 2 || h.dim == 3) && m.d.sectors && m.d.udf && m.d.Edf &&
-           h.nc > 0 && h.nc <= (h.dim == 2 ? kGroupCells : kGroupCells3) &&
-           (int)h.sectors.size() == (h.dim << h.dim) * h.dim;
-}
-
-template <int D>
-static cudaError_t launch_group_d(const std::vector<int> &ks, const soptx_mesh_s *const *ms, const double *const *rho,
-                                  const double *const *u, double *const *vals, double *const *dc, double *const *c,
-                                  cudaStream_t st)
-{
-    const int n = (int)ks.size();
-    for (int k0 = 0; k0 < n; k0 += kGroupMax) {
-        static thread_local LatGroup<D> G;   // ~24 KB: off the stack
-        G = LatGroup<D>{};
-        G.n = std::min(kGroupMax, n - k0);
-        for (int k = 0; k < G.n; k++) {
-            const int j = ks[k0 + k];
-            const soptx_mesh_s &m = *ms[j];
-            const auto &h = m.h;
-            LatReq<D> &R = G.r[k];
-            unsigned gen = ++m.lattice_gen;
-            if (gen == 0u) gen = ++m.lattice_gen;
-            R.nx = h.lat_n[0];
-            R.ny = h.lat_n[1];
-            R.nz = D == 3 ? h.lat_n[2] : 1;
-            constexpr int warps = 8 * kGroupCtas;
-            if (D == 2) {
-                // node chunks of 3 .. 48 for the cluster's warps
-                const int64_t groups = (h.nn + 2) / 3;
-                R.chunk = 3 * (int)std::max<int64_t>(1, std::min<int64_t>(16, groups / warps));
-            } else {
-                // even chunks of at most kChunk nodes, about as many per warp (as in the single step)
-                const int64_t rounds = (h.nn + warps * kChunk - 1) / (warps * kChunk);
-                int chunk = (int)std::max<int64_t>(1, (h.nn + warps * rounds - 1) / (warps * rounds));
-                R.chunk = chunk + (chunk & 1);
-            }
-            R.sgrid = lattice_sens_grid(h.nc);
-            R.gen = gen;
-            R.pbias = 0x38000000u + ((uint32_t)h.lat_kshift << 20);
-            R.nn = h.nn;
-            R.nc = h.nc;
-            R.ndof = h.ndof;
-            R.kscale = std::ldexp(1.0, h.lat_kshift);
-            R.sp = simp_params(m.mat);
-            R.B = sector_table<D>(h.sectors);
-            R.rho = rho[j];
-            R.u = u[j];
-            R.gscale = nullptr;
-            R.K0 = m.d.K0;
-            R.vals = vals[j];
-            R.dc = dc[j];
-            R.c = c[j];
-            R.partial = m.d.scratch;
-            R.Edf = (float2 *)m.d.Edf;
-            R.udf = m.d.udf;
-            R.node_off = m.d.node_off;
-            R.flag = m.d.lat_bad;
-            R.counter = m.d.counter;
-            R.kappa = (const float2 *)m.d.kappa;
-        }
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(G.n * kGroupCtas));
-        cfg.blockDim = dim3(256);
-        cfg.dynamicSmemBytes = 0;
-        cfg.stream = st;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = kGroupCtas;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        cudaError_t err = cudaLaunchKernelEx(&cfg, k_lattice_step_group<D>, G);
-        if (err != cudaSuccess) return err;
-    }
-    return cudaSuccess;
 }
 
 cudaError_t launch_lattice_group(const soptx_mesh_s *const *ms, const double *const *rho, const double *const *u,
