@@ -27,6 +27,13 @@ def _dptr(t, dtype, n, name):
     return ctypes.c_void_p(t.data_ptr())
 
 
+def _out(n, device):
+    """A new output and its address (nothing to check: a check costs about as much as the
+    allocation on the calls of small meshes)."""
+    t = torch.empty(n, dtype=torch.float64, device=device)
+    return t, t.data_ptr()
+
+
 def _hptr(t, n, name):
     if not isinstance(t, torch.Tensor) or t.is_cuda:
         raise TypeError("%s must be a host (CPU) tensor" % name)
@@ -109,34 +116,44 @@ class Mesh:
     # ------------------------------------------------------------ hot path
     def assemble_K(self, rho, vals=None, stream=None):
         if vals is None:
-            vals = torch.empty(self.nnz, dtype=torch.float64, device=self.device)
-        N.check(N.lib().soptx_assemble_K(self._h, _dptr(rho, torch.float64, self.n_cells, "rho"),
-                                         _dptr(vals, torch.float64, self.nnz, "vals"), _stream(stream)))
+            vals, pv = _out(self.nnz, self.device)
+        else:
+            pv = _dptr(vals, torch.float64, self.nnz, "vals")
+        N.check(N.lib().soptx_assemble_K(self._h, _dptr(rho, torch.float64, self.n_cells, "rho"), pv,
+                                         _stream(stream)))
         return vals
 
     def sensitivity(self, rho, u, dc=None, c=None, want_c=True, stream=None):
         if dc is None:
-            dc = torch.empty(self.n_cells, dtype=torch.float64, device=self.device)
+            dc, pd = _out(self.n_cells, self.device)
+        else:
+            pd = _dptr(dc, torch.float64, self.n_cells, "dc")
+        pc = None
         if want_c and c is None:
-            c = torch.empty(1, dtype=torch.float64, device=self.device)
+            c, pc = _out(1, self.device)
+        elif want_c:
+            pc = _dptr(c, torch.float64, 1, "c")
         N.check(N.lib().soptx_sensitivity(self._h, _dptr(rho, torch.float64, self.n_cells, "rho"),
-                                          _dptr(u, torch.float64, self.ndof, "u"),
-                                          _dptr(dc, torch.float64, self.n_cells, "dc"),
-                                          _dptr(c, torch.float64, 1, "c") if want_c else None, _stream(stream)))
+                                          _dptr(u, torch.float64, self.ndof, "u"), pd, pc, _stream(stream)))
         return dc, (c if want_c else None)
 
     def step(self, rho, u, vals=None, dc=None, c=None, stream=None):
         """K(rho), dc and c in one call (the per-iteration hot path)."""
         if vals is None:
-            vals = torch.empty(self.nnz, dtype=torch.float64, device=self.device)
+            vals, pv = _out(self.nnz, self.device)
+        else:
+            pv = _dptr(vals, torch.float64, self.nnz, "vals")
         if dc is None:
-            dc = torch.empty(self.n_cells, dtype=torch.float64, device=self.device)
+            dc, pd = _out(self.n_cells, self.device)
+        else:
+            pd = _dptr(dc, torch.float64, self.n_cells, "dc")
         if c is None:
-            c = torch.empty(1, dtype=torch.float64, device=self.device)
+            c, pc = _out(1, self.device)
+        else:
+            pc = _dptr(c, torch.float64, 1, "c")
         N.check(N.lib().soptx_assemble_and_sensitivity(
             self._h, _dptr(rho, torch.float64, self.n_cells, "rho"), _dptr(u, torch.float64, self.ndof, "u"),
-            _dptr(vals, torch.float64, self.nnz, "vals"), _dptr(dc, torch.float64, self.n_cells, "dc"),
-            _dptr(c, torch.float64, 1, "c"), _stream(stream)))
+            pv, pd, pc, _stream(stream)))
         return vals, dc, c
 
     def step_host(self, rho, u, vals=None, dcc=None, stream=None):
@@ -158,12 +175,11 @@ class Mesh:
         return vals, dcc[:self.n_cells], dcc[self.n_cells:]
 
     def compliance_vjp(self, rho, u, gout, want_u=True, stream=None):
-        grad_rho = torch.empty(self.n_cells, dtype=torch.float64, device=self.device)
-        grad_u = torch.empty(self.ndof, dtype=torch.float64, device=self.device) if want_u else None
+        grad_rho, pr = _out(self.n_cells, self.device)
+        grad_u, pu = _out(self.ndof, self.device) if want_u else (None, None)
         N.check(N.lib().soptx_compliance_vjp(
             self._h, _dptr(rho, torch.float64, self.n_cells, "rho"), _dptr(u, torch.float64, self.ndof, "u"),
-            _dptr(gout, torch.float64, 1, "gout"), _dptr(grad_rho, torch.float64, self.n_cells, "grad_rho"),
-            _dptr(grad_u, torch.float64, self.ndof, "grad_u") if want_u else None, _stream(stream)))
+            _dptr(gout, torch.float64, 1, "gout"), pr, pu, _stream(stream)))
         return grad_rho, grad_u
 
 
@@ -210,15 +226,12 @@ def step_group(meshes, rhos, us, stream=None):
     P = ctypes.c_void_p * max(n, 1)
     hm, pr, pu, pv, pd, pc = P(), P(), P(), P(), P(), P()
     for k, (m, rho, u) in enumerate(zip(meshes, rhos, us)):
-        vals = torch.empty(m.nnz, dtype=torch.float64, device=m.device)
-        dc = torch.empty(m.n_cells, dtype=torch.float64, device=m.device)
-        c = torch.empty(1, dtype=torch.float64, device=m.device)
+        vals, pv[k] = _out(m.nnz, m.device)
+        dc, pd[k] = _out(m.n_cells, m.device)
+        c, pc[k] = _out(1, m.device)
         hm[k] = m._h.value
         pr[k] = _dptr(rho, torch.float64, m.n_cells, "rho").value
         pu[k] = _dptr(u, torch.float64, m.ndof, "u").value
-        pv[k] = _dptr(vals, torch.float64, m.nnz, "vals").value
-        pd[k] = _dptr(dc, torch.float64, m.n_cells, "dc").value
-        pc[k] = _dptr(c, torch.float64, 1, "c").value
         outs.append((vals, dc, c))
     N.check(N.lib().soptx_assemble_and_sensitivity_group(n, hm, pr, pu, pv, pd, pc, _stream(stream)))
     return outs

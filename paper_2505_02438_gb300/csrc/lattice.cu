@@ -1070,8 +1070,7 @@ static cudaError_t launch_group_d(const std::vector<int> &ks, const soptx_mesh_s
 {
     const int n = (int)ks.size();
     for (int k0 = 0; k0 < n; k0 += kGroupMax) {
-        static thread_local LatGroup<D> G;   // ~24 KB: off the stack
-        G = LatGroup<D>{};
+        static thread_local LatGroup<D> G;   // ~24 KB: off the stack; its first n requests are read
         G.n = std::min(kGroupMax, n - k0);
         for (int k = 0; k < G.n; k++) {
             const int j = ks[k0 + k];
