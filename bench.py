@@ -892,9 +892,10 @@ def run_ours(args, rank, world, local_rank):
         "e2e": {"value": job_rate(nnz, world, n_e2e, e2e_ms) / 1e9, "unit": "GNNZ/s",
                 "h2d_bytes_per_step": 8 * (nc + ndof), "d2h_bytes_per_step": 8 * (nc + 1),
                 "steps": n_e2e},
-        # lattice: moduli (and u pairs), assembly, sensitivity (+ sum of c); general path: moduli and u pairs,
-        # fused gather, finalize (+ sum of c)
-        "gpu_launches": 3 * K,
+        # lattice: moduli (and u pairs), assembly, sensitivity (+ sum of c), small ones in one launch; meshes with
+        # strain-energy sensitivities: moduli, assembly, sensitivity; general path: moduli and u pairs, fused
+        # gather, finalize (+ sum of c)
+        "gpu_launches": (1 if mesh.path == "lattice" and nc <= (1536 if mesh.dim == 2 else 1024) else 3) * K,
         "wall_s_timed_region": wall,
     }
     if args.elem_prec == "fp32":

@@ -25,7 +25,7 @@
 // instruction also occupies the SM's FP64 pipe for 16 cycles, so only one lane tests the
 // residual and divides).  Per iteration, the general loop and this kernel: 60x20x4 Q1
 // hexahedra 20.2 and 9.8 us, 36x14x14 22.5 and 11.2, 60x20 Q1 quadrilaterals 14.6 and 8.0,
-// 160x60 18.3 and 9.8, 260x150 29.3 and 16; 4x2 19 and 11: where it fits it is the faster
+// 160x60 18.3 and 9.8, 260x150 29.3 and 16; 4x2 19 and 10: where it fits it is the faster
 // one.
 #include <algorithm>
 #include <cmath>

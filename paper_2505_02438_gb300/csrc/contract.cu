@@ -48,12 +48,12 @@ constexpr unsigned kFull = 0xffffffffu;
 // Per-cell record of the contraction (FP32): G row-major (G[m][i] = (J^-1)_{mi})
 // then |det J|, padded to whole float4s.
 template <int D> struct CGeo {
-    static constexpr int n4 = D == 3 ? 3 : 2;
+    static constexpr int n4 = 2;
 };
 // Reference integrals of one (a, b) pair in shared memory: M[k][l] padded to
 // whole float4s.
 template <int D> struct MPad {
-    static constexpr int n = D == 3 ? 12 : 4;
+    static constexpr int n = 4;
 };
 
 // The pair tables made at mesh creation.  Pairs come in tiles of 32, one per
@@ -121,32 +121,17 @@ __device__ __forceinline__ void contract_block(const float *M, const float *G, f
 template <int D>
 __device__ __forceinline__ void load_cgeo(const float4 *__restrict__ cg, int64_t e, float G[D * D], float &det)
 {
-    if (D == 3) {
-        const float4 g0 = __ldg(cg + 3 * e), g1 = __ldg(cg + 3 * e + 1), g2 = __ldg(cg + 3 * e + 2);
-        G[0] = g0.x; G[1] = g0.y; G[2] = g0.z; G[3] = g0.w;
-        G[4] = g1.x; G[5] = g1.y; G[6] = g1.z; G[7] = g1.w;
-        G[8] = g2.x;
-        det = g2.y;
-    } else {
-        const float4 g0 = __ldg(cg + 2 * e), g1 = __ldg(cg + 2 * e + 1);
-        G[0] = g0.x; G[1] = g0.y; G[2] = g0.z; G[3] = g0.w;
-        det = g1.x;
-    }
+    const float4 g0 = __ldg(cg + 2 * e), g1 = __ldg(cg + 2 * e + 1);
+    G[0] = g0.x; G[1] = g0.y; G[2] = g0.z; G[3] = g0.w;
+    det = g1.x;
 }
 
 template <int D>
 __device__ __forceinline__ void load_mpair(const float *Ms, int pair, float M[D * D])
 {
     const float4 *p = reinterpret_cast<const float4 *>(Ms + pair * MPad<D>::n);
-    if (D == 3) {
-        const float4 a = p[0], b = p[1], c = p[2];
-        M[0] = a.x; M[1] = a.y; M[2] = a.z; M[3] = a.w;
-        M[4] = b.x; M[5] = b.y; M[6] = b.z; M[7] = b.w;
-        M[8] = c.x;
-    } else {
-        const float4 a = p[0];
-        M[0] = a.x; M[1] = a.y; M[2] = a.z; M[3] = a.w;
-    }
+    const float4 a = p[0];
+    M[0] = a.x; M[1] = a.y; M[2] = a.z; M[3] = a.w;
 }
 
 // Accumulate x into the unnormalised pair (s, c).
@@ -472,15 +457,8 @@ __global__ void __launch_bounds__(256, D == 2 ? 4 : 3) k_contract_pairs(const Pa
                 } else if (k < cnt) {
                     bad |= isnan(cur.E.y);
                     float G[D * D], det;
-                    if (D == 3) {
-                        G[0] = cur.g[0].x; G[1] = cur.g[0].y; G[2] = cur.g[0].z; G[3] = cur.g[0].w;
-                        G[4] = cur.g[1].x; G[5] = cur.g[1].y; G[6] = cur.g[1].z; G[7] = cur.g[1].w;
-                        G[8] = cur.g[2].x;
-                        det = cur.g[2].y;
-                    } else {
-                        G[0] = cur.g[0].x; G[1] = cur.g[0].y; G[2] = cur.g[0].z; G[3] = cur.g[0].w;
-                        det = cur.g[1].x;
-                    }
+                    G[0] = cur.g[0].x; G[1] = cur.g[0].y; G[2] = cur.g[0].z; G[3] = cur.g[0].w;
+                    det = cur.g[1].x;
                     float M[D * D], K[D][D];
                     load_mpair<D>(Ms, m0, M);
                     contract_block<D>(M, G, det, A.lam, A.mu, K);
