@@ -188,15 +188,16 @@ def traffic_record(kernel_file, kernel_name, workload, prec="fp64"):
     `prec`) from the committed ncu summary, valid only while the kernel source
     is unchanged (kernel_source_sha matches)."""
     src = os.path.join(ROOT, "paper_2505_02438_gb300", "csrc", kernel_file)
-    rec = os.path.join(ROOT, "profiles", "traffic.txt")
-    if not (os.path.exists(src) and os.path.exists(rec)):
+    if not os.path.exists(src):
         return None
     h = kernel_source_sha(kernel_file)
-    for line in open(rec):
-        kv = dict(x.split("=", 1) for x in line.split() if "=" in x)
-        if kv.get("kernel") == kernel_name and kv.get("source_sha") == h and kv.get("workload") == workload \
-                and kv.get("prec", "fp64") == prec:
-            return float(kv["dram_bytes_per_launch"])
+    for name in ("traffic.txt", "traffic_block_rows.txt"):
+        rec = os.path.join(ROOT, "profiles", name)
+        for line in open(rec) if os.path.exists(rec) else ():
+            kv = dict(x.split("=", 1) for x in line.split() if "=" in x)
+            if kv.get("kernel") == kernel_name and kv.get("source_sha") == h and kv.get("workload") == workload \
+                    and kv.get("prec", "fp64") == prec:
+                return float(kv["dram_bytes_per_launch"])
     return None
 
 
