@@ -55,6 +55,7 @@
 //            of the transpose (0xffff: none) | row length << 16 | (cells(5-6) | lg lanes << 2) << 27
 //   records: [rows][32] 16 bits: cell of the chunk (cell_bits) | (a nb + b) << cell_bits
 #include <algorithm>
+#include <cfloat>
 #include <cstdint>
 
 #include "df64.cuh"
@@ -161,6 +162,14 @@ __device__ __forceinline__ df times(df E, float k)
 {
     const float p = __fmul_rn(E.h, k);
     return df{p, __fmaf_rn(E.l, k, __fmaf_rn(E.h, k, -p))};
+}
+
+// max that keeps a NaN
+__device__ __forceinline__ float max_nan(float a, float b)
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
 }
 
 // The FP32 block of a pair and cell: P = |det J| G^T M G, K = lam P + mu P^T + mu tr P I.
@@ -502,6 +511,13 @@ __global__ void __launch_bounds__(32 * (W + 1), MINB) k_block_rows(const BlockAr
                     }
                 }
             }
+            // the largest head of the block (NaN when one is): beyond the floats it is redone
+            // in FP64 too; below kRebiasMin the fast conversion would add up to 2^-126 to
+            // entries that are not far above it
+            float big = 0.f;
+#pragma unroll
+            for (int p = 0; p < 9; p++) big = max_nan(big, fabsf(v[p].x));
+            bad |= !(big <= FLT_MAX);
             if (!free) {
                 if (!mbar_wait(&s_free[s], (k >> 1) & 1)) return give_up();
                 free = true;
@@ -515,6 +531,9 @@ __global__ void __launch_bounds__(32 * (W + 1), MINB) k_block_rows(const BlockAr
                     block_fp64<SRC>(A, B, Ms, rec, pairs + 32 * t + lane, 1 << lg, acc);
 #pragma unroll
                     for (int p = 0; p < 9; p++) dv[p] = acc[p];
+                } else if (big < kRebiasMin) {
+#pragma unroll
+                    for (int p = 0; p < 9; p++) dv[p] = (double)v[p].x + (double)v[p].y;
                 } else {
 #pragma unroll
                     for (int p = 0; p < 9; p++) dv[p] = pair_to_double_rebias(v[p].x, v[p].y);

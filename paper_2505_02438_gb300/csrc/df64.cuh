@@ -177,7 +177,10 @@ __device__ __forceinline__ double pair_to_double(float s, float c)
 
 // The same in 13 instructions: the halves are widened by a sign-extending shift
 // and an exponent rebias without a test for zero or denormal floats, which turn
-// into values below 2^-126; only s = c = 0 is set to zero again.
+// into values below 2^-126; only s = c = 0 is set to zero again.  Correctly rounded
+// for |s| >= kRebiasMin (2^-126 is then below half a unit of the result's last place)
+// and finite s; callers convert smaller values otherwise.
+constexpr float kRebiasMin = 0x1p-72f;
 __device__ __forceinline__ double pair_to_double_rebias(float s, float c)
 {
     const int a = __float_as_int(s), b = __float_as_int(c);
