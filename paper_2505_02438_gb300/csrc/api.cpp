@@ -36,7 +36,7 @@ static void free_device(DeviceMesh &d)
     void *ptrs[] = {d.indptr, d.indices, d.cell_node, d.node_off, d.inc_ptr, d.inc,
                     d.pos, d.geo, d.M, d.K, d.scratch, d.Edf, d.kappa, d.K0, d.sectors, d.udf, d.part,
                     d.inc_e, d.inc_a, d.counter, d.xcell, d.qw, d.qdphi, d.qdgeo, d.cg, d.lat_bad, d.stage,
-                    d.kvals, d.sgeo, d.sq, d.ssf, d.cgeo, d.Mf, d.ptoff, d.pia, d.pib, d.pmeta, d.pre, d.prm, d.pblk,
+                    d.kvals, d.sgeo, d.gtab, d.sq, d.ssf, d.cgeo, d.Mf, d.ptoff, d.pia, d.pib, d.pmeta, d.pre, d.prm, d.pblk,
                     d.bblob, d.bcoff, d.bcell, d.bM, d.bkblk, d.cticket, d.rbuf};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -105,7 +105,41 @@ static float2 split_pair(double x)
     return make_float2(hh, (float)(x - (double)hh));
 }
 
-// Tables of the strain-energy sensitivities (k_strain_energy).
+// General cells (strain_general.cu): the geometry of every Gauss point, computed on the
+// device, and the tables of orders 2 and 3.
+static soptx_status setup_strain_general(soptx_mesh_s &m, const RefElement &ref, cudaStream_t st)
+{
+    const HostMesh &h = m.h;
+    std::vector<double> tab;
+    if (h.order > 1) {
+        std::vector<double> w1, val, der;
+        tensor_1d_factors(h.order, w1, val, der);
+        const int n = h.order + 1;
+        tab = val;
+        tab.insert(tab.end(), der.begin(), der.end());
+        for (int a = 0; a < h.nb; a++) {
+            const int *la = ref.lat[(size_t)a].data();
+            tab.push_back(la[0] + n * la[1] + (h.dim == 3 ? n * n * la[2] : 0));
+        }
+    }
+    soptx_status s = tab.empty() ? SOPTX_OK : upload(&m.d.gtab, tab, st, m.device_bytes, "tables of the Gauss points");
+    if (s != SOPTX_OK) return s;
+    m.d.snq = m.d.nq;
+    const size_t bytes = (size_t)h.nc * m.d.snq * (h.dim * h.dim + 1) * sizeof(float2);
+    cudaError_t e = dev_alloc((void **)&m.d.sgeo, bytes);
+    if (e == cudaSuccess) e = launch_point_geometry(m, st);
+    // (the host table goes out of scope: its copy has to be done)
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return cuda_status(e, "point geometry");
+    }
+    m.device_bytes += (int64_t)bytes;
+    m.d.strain = true;
+    return SOPTX_OK;
+}
+
+// Tables of the strain-energy sensitivities of affine cells (k_strain_energy).
 static soptx_status setup_strain(soptx_mesh_s &m, const RefElement &ref, cudaStream_t st)
 {
     const HostMesh &h = m.h;
@@ -117,10 +151,10 @@ static soptx_status setup_strain(soptx_mesh_s &m, const RefElement &ref, cudaStr
     for (size_t t = 0; t < q.dphi.size(); t++) tab[q.nq + t] = split_pair(q.dphi[t]);
     const int ng = h.dim * h.dim + 1;
     const int64_t ncg = m.path == SOPTX_PATH_UNIFORM ? 1 : h.nc;
-    std::vector<float2> sg(h.nonaffine ? 0 : (size_t)ncg * ng);
+    std::vector<float2> sg((size_t)ncg * ng);
     for (size_t t = 0; t < sg.size(); t++) sg[t] = split_pair(h.geo[t]);
     soptx_status s = upload(&m.d.sq, tab, st, m.device_bytes, "quadrature table");
-    if (s == SOPTX_OK && !h.nonaffine) s = upload(&m.d.sgeo, sg, st, m.device_bytes, "cell geometry pairs");
+    if (s == SOPTX_OK) s = upload(&m.d.sgeo, sg, st, m.device_bytes, "cell geometry pairs");
     if (s == SOPTX_OK && h.dim == 3 && !is_simplex(h.cell) && (h.order == 2 || h.order == 3)) {
         // the 1D factors of the tensor rule, for the sum-factorised kernel
         std::vector<double> w1, val, der;
@@ -136,20 +170,10 @@ static soptx_status setup_strain(soptx_mesh_s &m, const RefElement &ref, cudaStr
         }
         s = upload(&m.d.ssf, sf, st, m.device_bytes, "1D factors of the rule");
     }
-    m.d.snq = q.nq;
-    if (s == SOPTX_OK && h.nonaffine) {
-        // general cells: the geometry of every point, computed on the device
-        const size_t bytes = (size_t)h.nc * q.nq * ng * sizeof(float2);
-        cudaError_t e = dev_alloc((void **)&m.d.sgeo, bytes);
-        if (e == cudaSuccess) e = launch_point_geometry(m, st);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            s = cuda_status(e, "point geometry");
-        } else {
-            m.device_bytes += (int64_t)bytes;
-        }
+    if (s == SOPTX_OK) {
+        m.d.snq = q.nq;
+        m.d.strain = true;
     }
-    if (s == SOPTX_OK) m.d.strain = true;
     return s;
 }
 
@@ -766,7 +790,7 @@ soptx_status soptx_mesh_create(int dim, soptx_cell cell, int order, int64_t n_ve
         // the weights and reference gradients of the rule); general cells at the
         // points of the rule that defines their FP64 element matrices (FP32 ones keep
         // the gather: their sensitivities are those of the rounded matrices)
-        s = setup_strain(*m, ref, st);
+        s = h.nonaffine ? setup_strain_general(*m, ref, st) : setup_strain(*m, ref, st);
         // 2D: FP32 element matrices contracted per call, the cache not read; FP64 ones
         // and a uniform mesh's one matrix: the pair kernel reads each node pair's
         // blocks once for both row blocks

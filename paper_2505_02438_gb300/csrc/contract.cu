@@ -592,10 +592,6 @@ struct StrainArgs {
     SimpParams sp;
     const float2 *__restrict__ geo;   // [nc or 1][d*d + 1] G row-major, |det J|, as pairs
     int64_t geo_stride;               // d*d + 1, or 0 when every cell has the same Jacobian
-    // general bilinear / trilinear cells: G and w |det J| at every point, entry t of
-    // point q of cell e at geo[e geo_stride + (q (d*d + 1) + t) geo_step]
-    bool general;
-    int64_t geo_step;
     const float2 *__restrict__ qw;    // [nq] weights
     const float2 *__restrict__ qd;    // [nq][nb][d] reference gradients
     float2 lam, mu;                   // Lame constants at E = 1, as pairs
@@ -611,9 +607,7 @@ struct StrainArgs {
 // <= 256 (the grid sum of c).
 // NBT = the cell's node count, so the staging loads of a cell issue together,
 // or 0 for any count (runtime loops).
-// GEN: general cells, the geometry of every point read as it is needed (det then
-// holds w |det J|).
-template <int D, bool PAIR, int NBT, bool GEN = false>
+template <int D, bool PAIR, int NBT>
 __global__ void __launch_bounds__(128) k_strain_energy(const StrainArgs A)
 {
     using S = SArith<PAIR>;
@@ -651,18 +645,11 @@ __global__ void __launch_bounds__(128) k_strain_energy(const StrainArgs A)
             }
             V G[D * D], det;
             const float2 *gp = A.geo + e * A.geo_stride;
-            auto load_geo = [&]() {
 #pragma unroll
-                for (int t = 0; t < D * D; t++) G[t] = S::from_pair(gp[t * (GEN ? A.geo_step : 1)]);
-                det = S::from_pair(gp[D * D * (GEN ? A.geo_step : 1)]);
-            };
-            if (!GEN) load_geo();
+            for (int t = 0; t < D * D; t++) G[t] = S::from_pair(gp[t]);
+            det = S::from_pair(gp[D * D]);
             typename S::Acc s;
             for (int q = 0; q < nq; q++) {
-                if (GEN) {
-                    load_geo();
-                    gp += (D * D + 1) * A.geo_step;
-                }
                 typename S::Acc U[D][D];
                 const float2 *dq = A.qd + (size_t)q * nb * D;
 #pragma unroll 2
@@ -705,9 +692,9 @@ __global__ void __launch_bounds__(128) k_strain_energy(const StrainArgs A)
                 typename S::Acc dens;
                 S::fma(dens, lam, S::mul(tr, tr));
                 S::fma(dens, mu, S::val(sh));
-                S::fma(s, GEN ? det : S::from_pair(__ldg(A.qw + q)), S::val(dens));
+                S::fma(s, S::from_pair(__ldg(A.qw + q)), S::val(dens));
             }
-            const double sd = S::to_double(GEN ? S::val(s) : S::mul(S::val(s), det));
+            const double sd = S::to_double(S::mul(S::val(s), det));
             const double r = A.rho[e];
             A.out[e] = g * simp_dE(A.sp, r) * sd;
             mine += simp_E(A.sp, r) * sd;
@@ -718,7 +705,7 @@ __global__ void __launch_bounds__(128) k_strain_energy(const StrainArgs A)
 
 // The strain energy density at quadrature point q of a cell whose
 // displacements are staged at us[(b d + i) * ustride] (reference gradients at
-// the point dq[b][m], G row-major).
+// the point dq[b][m], G row-major), times the point's weight.
 template <int D, bool PAIR>
 __device__ __forceinline__ typename SArith<PAIR>::V
 point_energy(const StrainArgs &A, const typename SArith<PAIR>::V *us, int ustride, int q,
@@ -765,7 +752,7 @@ point_energy(const StrainArgs &A, const typename SArith<PAIR>::V *us, int ustrid
     typename S::Acc dens;
     S::fma(dens, lam, S::mul(tr, tr));
     S::fma(dens, mu, S::val(sh));
-    return S::val(dens);
+    return S::mul(S::from_pair(__ldg(A.qw + q)), S::val(dens));
 }
 
 // The same sensitivities with a warp per cell, for cells with many nodes and
@@ -797,22 +784,13 @@ __global__ void __launch_bounds__(128) k_strain_energy_warp(const StrainArgs A)
         const float2 *gp = A.geo + e * A.geo_stride;
 #pragma unroll
         for (int t = 0; t < D * D; t++) G[t] = S::from_pair(gp[t]);
-        V det = S::from_pair(gp[D * D]);
+        const V det = S::from_pair(gp[D * D]);
         V sv = S::from_pair(make_float2(0.f, 0.f));
-        for (int q = lane; q < A.nq; q += 32) {
-            if (A.general) {
-                const float2 *gq = gp + q * (D * D + 1);
-#pragma unroll
-                for (int t = 0; t < D * D; t++) G[t] = S::from_pair(gq[t]);
-                det = S::from_pair(gq[D * D]);
-            }
-            const V en = point_energy<D, PAIR>(A, us, 1, q, G, lam, mu);
-            sv = S::sum(sv, S::mul(A.general ? det : S::from_pair(__ldg(A.qw + q)), en));
-        }
+        for (int q = lane; q < A.nq; q += 32) sv = S::sum(sv, point_energy<D, PAIR>(A, us, 1, q, G, lam, mu));
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sv = S::sum(sv, S::shfl_xor(sv, o));
         if (lane == 0) {
-            const double sd = S::to_double(A.general ? sv : S::mul(sv, det));
+            const double sd = S::to_double(S::mul(sv, det));
             const double r = A.rho[e];
             A.out[e] = g * simp_dE(A.sp, r) * sd;
             mine += simp_E(A.sp, r) * sd;
@@ -928,7 +906,7 @@ __global__ void __launch_bounds__(128) k_strain_hex_sf(const StrainArgs A, const
         const float2 *gp = A.geo + e * A.geo_stride;
 #pragma unroll
         for (int t = 0; t < D * D; t++) G[t] = S::from_pair(gp[t]);
-        V det = S::from_pair(gp[D * D]);
+        const V det = S::from_pair(gp[D * D]);
         // third index at each point q1 + n q2 + n2 q3, and the density there
         V sv = S::from_pair(make_float2(0.f, 0.f));
         for (int p = lane; p < n3; p += 32) {
@@ -948,19 +926,13 @@ __global__ void __launch_bounds__(128) k_strain_hex_sf(const StrainArgs A, const
                 Uv[i][1] = S::val(d2);
                 Uv[i][2] = S::val(d3);
             }
-            if (A.general) {
-                const float2 *gq = gp + p * (D * D + 1);
-#pragma unroll
-                for (int t = 0; t < D * D; t++) G[t] = S::from_pair(gq[t]);
-                det = S::from_pair(gq[D * D]);
-            }
-            const V w = A.general ? det : S::mul(S::mul(s_w[q1], s_w[q2]), s_w[q3]);
+            const V w = S::mul(S::mul(s_w[q1], s_w[q2]), s_w[q3]);
             sv = S::sum(sv, S::mul(w, density_from_grad<D, PAIR>(Uv, G, lam, mu)));
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sv = S::sum(sv, S::shfl_xor(sv, o));
         if (lane == 0) {
-            const double sd = S::to_double(A.general ? sv : S::mul(sv, det));
+            const double sd = S::to_double(S::mul(sv, det));
             const double r = A.rho[e];
             A.out[e] = g * simp_dE(A.sp, r) * sd;
             mine += simp_E(A.sp, r) * sd;
@@ -968,135 +940,6 @@ __global__ void __launch_bounds__(128) k_strain_hex_sf(const StrainArgs A, const
     }
     if (A.c) grid_sum_last_block(mine, A.partial, A.counter, A.c);
 }
-
-// General trilinear hexahedra of order 1 (float pairs), one thread per cell.  The
-// eight Gauss points are the corners of a cube, so the reference displacement
-// gradient at all of them is a Walsh transform each way: with the differences (bit
-// set) and sums (bit clear) of the corner values along the axes, w_b, and a =
-// 1 / sqrt(3), the derivative along axis 1 at the signs (s2, s3) is
-//     (w_100 + s2 a w_110 + s3 a w_101 + s2 s3 a^2 w_111) / 4
-// (and so on), about 150 float-pair sums in place of 576 multiply-adds; the 1 / 16
-// of the energy is applied at the end.  u is read from the cell's nodes, the
-// geometry of the points (80 bytes each) in planes over the cells: 123 MB for
-// 192,000 cells, which bounds the kernel.  (In the gather over the cached element
-// matrices, fused with the assembly, the sensitivities took 340 us on the jittered
-// 120x40x40 hexahedra.)
-__global__ void __launch_bounds__(128, 5) k_strain_hex8(const StrainArgs A)
-{
-    using S = SArith<true>;
-    // derivative along axis m of component i at the signs s of the other two axes (the
-    // lower axis in bit 0), times 4, at us[((3 m + i) 4 + s) 128 + thread]: in registers,
-    // with the eight points unrolled, the kernel waited on instruction fetches (80 us)
-    __shared__ float2 us[36 * 128];
-    const int tid = threadIdx.x;
-    const double g = A.gscale ? *A.gscale : -1.0;
-    const df lam = S::from_pair(A.lam), mu = S::from_pair(A.mu);
-    const df a1 = df_from_double(0.57735026918962576451), a2 = df_from_double(1.0 / 3.0);
-    double mine = 0.0;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + tid; e < A.nc; e += (int64_t)gridDim.x * blockDim.x) {
-        int32_t nd[8];
-#pragma unroll
-        for (int b = 0; b < 8; b++) nd[b] = __ldg(A.cell_node + e * 8 + b);
-#pragma unroll 1
-        for (int i = 0; i < 3; i++) {
-            df w[8];
-#pragma unroll
-            for (int b = 0; b < 8; b++) w[b] = S::from_u(__ldg(A.u + 3 * (int64_t)nd[b] + i));
-#pragma unroll
-            for (int m = 0; m < 3; m++)
-#pragma unroll
-                for (int b = 0; b < 8; b++)
-                    if (!(b & (1 << m))) {
-                        const df lo = w[b], hi = w[b | (1 << m)];
-                        w[b] = df_add_lazy(lo, hi);
-                        w[b | (1 << m)] = df_add_lazy(hi, df_neg(lo));
-                    }
-            w[3] = df_mul(w[3], a1);
-            w[5] = df_mul(w[5], a1);
-            w[6] = df_mul(w[6], a1);
-            w[7] = df_mul(w[7], a2);
-#pragma unroll
-            for (int m = 0; m < 3; m++) {
-                const int p = m == 0 ? 1 : 0, r = m == 2 ? 1 : 2;   // the other axes
-                const df c0 = w[1 << m], cp = w[1 << m | 1 << p], cr = w[1 << m | 1 << r], cc = w[7];
-                const df pl = df_add_lazy(c0, df_neg(cp)), ph = df_add_lazy(c0, cp);
-                const df ql = df_add_lazy(cr, df_neg(cc)), qh = df_add_lazy(cr, cc);
-                float2 *o = us + (3 * m + i) * 4 * 128 + tid;
-                const df v[4] = {df_add_lazy(pl, df_neg(ql)), df_add_lazy(ph, df_neg(qh)), df_add_lazy(pl, ql),
-                                 df_add_lazy(ph, qh)};
-#pragma unroll
-                for (int k = 0; k < 4; k++) o[k * 128] = make_float2(v[k].h, v[k].l);
-            }
-        }
-        S::Acc s;
-        const float2 *gp = A.geo + e;
-#pragma unroll 1
-        for (int q = 0; q < 8; q++, gp += 10 * A.geo_step) {
-            df G[9], Uv[3][3];
-#pragma unroll
-            for (int t = 0; t < 9; t++) G[t] = S::from_pair(__ldcs(gp + t * A.geo_step));
-            const df wd = S::from_pair(__ldcs(gp + 9 * A.geo_step));
-            const int k[3] = {q >> 1, (q & 1) | ((q >> 2) << 1), q & 3};
-#pragma unroll
-            for (int i = 0; i < 3; i++)
-#pragma unroll
-                for (int m = 0; m < 3; m++) Uv[i][m] = S::from_pair(us[((3 * m + i) * 4 + k[m]) * 128 + tid]);
-            S::fma(s, wd, density_from_grad<3, true>(Uv, G, lam, mu));
-        }
-        const double sd = 0.0625 * S::to_double(S::val(s));
-        const double r = A.rho[e];
-        A.out[e] = g * simp_dE(A.sp, r) * sd;
-        mine += simp_E(A.sp, r) * sd;
-    }
-    if (A.c) grid_sum_last_block(mine, A.partial, A.counter, A.c);
-}
-
-// At mesh creation: G = J^-1 and w |det J| of general cells at the Gauss points, in
-// FP64, stored as float pairs.
-template <int D>
-__global__ void k_point_geometry(int64_t nc, int nq, const double *__restrict__ xcell, const double *__restrict__ qw,
-                                 const double *__restrict__ dgeo, int64_t stride, int64_t step, float2 *__restrict__ geo)
-{
-    constexpr int NV = 1 << D;
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nc * nq; x += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t e = x / nq;
-        const int q = (int)(x - e * nq);
-        const double *xv = xcell + e * NV * D;
-        double J[D][D] = {};   // from the edge vectors: the rounding does not grow with the cell's distance from the origin
-        for (int v = 1; v < NV; v++)
-            for (int i = 0; i < D; i++)
-                for (int m = 0; m < D; m++) J[i][m] += (xv[v * D + i] - xv[i]) * dgeo[(q * NV + v) * D + m];
-        double G[D * D], det;
-        if constexpr (D == 2) {
-            det = J[0][0] * J[1][1] - J[0][1] * J[1][0];
-            G[0] = J[1][1] / det;
-            G[1] = -J[0][1] / det;
-            G[2] = -J[1][0] / det;
-            G[3] = J[0][0] / det;
-        } else {
-            double C[3][3];   // cofactors
-            for (int i = 0; i < 3; i++)
-                for (int m = 0; m < 3; m++) {
-                    const int i1 = (i + 1) % 3, i2 = (i + 2) % 3, m1 = (m + 1) % 3, m2 = (m + 2) % 3;
-                    C[i][m] = J[i1][m1] * J[i2][m2] - J[i1][m2] * J[i2][m1];
-                }
-            det = J[0][0] * C[0][0] + J[0][1] * C[0][1] + J[0][2] * C[0][2];
-            for (int i = 0; i < 3; i++)
-                for (int m = 0; m < 3; m++) G[m * 3 + i] = C[i][m] / det;
-        }
-        float2 *o = geo + e * stride + (int64_t)q * (D * D + 1) * step;
-        auto put = [&](int t, double v) {
-            const float h = __double2float_rn(v);
-            o[t * step] = make_float2(h, __double2float_rn(v - (double)h));
-        };
-        for (int t = 0; t < D * D; t++) put(t, G[t]);
-        put(D * D, qw[q] * fabs(det));
-    }
-}
-
-// One thread per cell reads the geometry of general cells in planes over the cells,
-// a warp per cell point after point.
-bool point_planes(const soptx_mesh_s &m) { return !m.d.ssf && (int64_t)m.h.nb * m.d.snq < 256; }
 
 template <int D, bool CACHED, bool UNIF>
 cudaError_t pairs_launch(const soptx_mesh_s &m, const double *rho, double *vals, cudaStream_t st)
@@ -1195,25 +1038,12 @@ cudaError_t launch_contract_assemble(const soptx_mesh_s &m, const double *rho, d
                          : pairs_launch<2, false, false>(m, rho, vals, st);
 }
 
-cudaError_t launch_point_geometry(const soptx_mesh_s &m, cudaStream_t st)
-{
-    const auto &h = m.h;
-    const int ng = h.dim * h.dim + 1;
-    const bool pl = point_planes(m);
-    const int64_t stride = pl ? 1 : (int64_t)m.d.snq * ng, step = pl ? h.nc : 1;
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((h.nc * m.d.snq + 255) / 256, 152 * 16));
-    if (h.dim == 2)
-        k_point_geometry<2><<<grid, 256, 0, st>>>(h.nc, m.d.snq, m.d.xcell, m.d.qw, m.d.qdgeo, stride, step, m.d.sgeo);
-    else
-        k_point_geometry<3><<<grid, 256, 0, st>>>(h.nc, m.d.snq, m.d.xcell, m.d.qw, m.d.qdgeo, stride, step, m.d.sgeo);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_strain_sensitivity(const soptx_mesh_s &m, const double *rho, const double *u, double *out,
                                       double *c, const double *gscale, cudaStream_t st, int max_grid)
 {
     const auto &h = m.h;
     if (h.nc == 0) return c ? cudaMemsetAsync(c, 0, sizeof(double), st) : cudaSuccess;
+    if (h.nonaffine) return launch_general_sensitivity(m, rho, u, out, c, gscale, st, max_grid);
     StrainArgs A;
     A.nc = h.nc;
     A.nb = h.nb;
@@ -1224,13 +1054,6 @@ cudaError_t launch_strain_sensitivity(const soptx_mesh_s &m, const double *rho, 
     A.sp = simp_params(m.mat);
     A.geo = m.d.sgeo;
     A.geo_stride = m.path == SOPTX_PATH_UNIFORM ? 0 : h.dim * h.dim + 1;
-    A.general = h.nonaffine;
-    A.geo_step = 1;
-    if (A.general) {
-        const bool pl = point_planes(m);
-        A.geo_stride = pl ? 1 : (int64_t)m.d.snq * (h.dim * h.dim + 1);
-        A.geo_step = pl ? h.nc : 1;
-    }
     A.qw = m.d.sq;
     A.qd = m.d.sq + m.d.snq;
     auto pair = [](double x) {
@@ -1270,12 +1093,6 @@ cudaError_t launch_strain_sensitivity(const soptx_mesh_s &m, const double *rho, 
         k<<<(int)grid, 128, smem, st>>>(A);
         return cudaGetLastError();
     }
-    if (A.general && h.dim == 3) {   // order 1
-        int64_t grid = std::max<int64_t>(1, std::min<int64_t>((h.nc + 127) / 128, m.d.scratch_len));
-        if (max_grid > 0) grid = std::min<int64_t>(grid, max_grid);
-        k_strain_hex8<<<(int)grid, 128, 0, st>>>(A);
-        return cudaGetLastError();
-    }
     // threads per block: a power of two whose staging fits in 96 KiB
     int T = 128;
     while (T > 32 && (size_t)T * h.nb * h.dim * vb > 96 * 1024) T >>= 1;
@@ -1283,8 +1100,6 @@ cudaError_t launch_strain_sensitivity(const soptx_mesh_s &m, const double *rho, 
     int64_t grid = std::max<int64_t>(1, std::min<int64_t>((h.nc + T - 1) / T, m.d.scratch_len));
     if (max_grid > 0) grid = std::min<int64_t>(grid, max_grid);
     void (*k)(StrainArgs) = nullptr;
-    if (A.general)   // bilinear quadrilaterals of order 1 and 2 (FP64 element matrices)
-        k = h.nb == 4 ? k_strain_energy<2, true, 4, true> : k_strain_energy<2, true, 9, true>;
 #define SOPTX_SE(DD, NBB)                                                                                     \
     if (h.dim == DD && (NBB == 0 || h.nb == NBB) && !k)                                                      \
         k = f32 ? k_strain_energy<DD, false, NBB> : k_strain_energy<DD, true, NBB>;

@@ -143,11 +143,12 @@ struct DeviceMesh {
     // general path
     float2 *udf = nullptr;         // [ndof] u as float pairs (general path; lattice: one-call step)
     double *part = nullptr;        // [nc][nb] per-(cell, node) partials of u_e^T K_e^0 u_e
-    // meshes of affine cells, general cells with FP64 element matrices: strain-energy
-    // sensitivities (contract.cu)
-    bool strain = false;           // the sensitivities take k_strain_energy
+    // meshes of affine cells (contract.cu), general cells with FP64 element matrices
+    // (strain_general.cu): strain-energy sensitivities
+    bool strain = false;           // the sensitivities take one of their kernels
     float2 *sgeo = nullptr;        //   [nc, or 1 when uniform][d*d + 1] G and |det J| as float pairs;
-                                   //   general cells: G and w |det J| at every point (StrainArgs)
+                                   //   general cells: G and w |det J| at every point (GeneralArgs)
+    double *gtab = nullptr;        //   general cells of order 2, 3: tables (GeneralArgs)
     float2 *sq = nullptr;          //   quadrature: weights [snq], reference gradients [snq][nb][d]
     int snq = 0;
     float2 *ssf = nullptr;         //   hexahedra of order 2, 3: 1D weights, basis values and derivatives,
@@ -272,7 +273,10 @@ bool contract_fits(int dim, int nb, int max_deg);
 bool pairs_fit(int dim, int nb, int max_deg);
 cudaError_t launch_contract_assemble(const soptx_mesh_s &m, const double *rho, double *vals, cudaStream_t st);
 cudaError_t launch_pair_blocks(const soptx_mesh_s &m, int64_t nrec, cudaStream_t st);
+// strain_general.cu
 cudaError_t launch_point_geometry(const soptx_mesh_s &m, cudaStream_t st);
+cudaError_t launch_general_sensitivity(const soptx_mesh_s &m, const double *rho, const double *u, double *out,
+                                       double *c, const double *gscale, cudaStream_t st, int max_grid);
 // max_grid > 0 caps the blocks (the kernel loops over the cells): beside a
 // persistent assembly, a block per SM leaves it the rest of the GPU
 cudaError_t launch_strain_sensitivity(const soptx_mesh_s &m, const double *rho, const double *u, double *out,
