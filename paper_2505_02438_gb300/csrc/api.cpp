@@ -537,6 +537,16 @@ static soptx_status setup_block_rows(soptx_mesh_s &m, const RefElement &ref, con
     L.sym = m.prec == SOPTX_ELEM_FP64;
     // lanes that read the same block of K^0 beside one another (Q3 box 26x9x9: 202 -> 197 us)
     L.by_code = src == kBlockUniform;
+    if (nb == 4) {
+        // linear tetrahedra meet 24 cells a node and 14 blocks: at the limits of the others
+        // a chunk has 7 nodes and the data-moving warp is the bottleneck (assembly of 1.1 M
+        // cells FP32 383 us, FP64 409; node-owner kernel before it 242 in FP32).  FP64: larger
+        // chunks, 289 (320 blocks and 300 cells 281, but slower than these below 100,000
+        // cells).  FP32: four CTAs of four warps, each with a data-moving warp, 250 us
+        // (100 blocks 273, three CTAs 260, two with 256 blocks 289)
+        L.blocks = src == kBlockContract ? 128 : 256;
+        L.cells = src == kBlockContract ? 140 : 256;
+    }
     BlockTables T;
     if (!build_block_tables(h, coords, cv, L, T)) return SOPTX_OK;
     const int64_t smem = block_smem(src, nb, T);

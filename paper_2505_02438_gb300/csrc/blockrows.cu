@@ -663,6 +663,7 @@ cudaError_t launch_block_rows(const soptx_mesh_s &m, const double *rho, double *
 {
     cudaError_t err = launch_prep(m, rho, nullptr, st);
     if (err != cudaSuccess || m.d.bchunks == 0) return err;
+    if (m.d.bsrc == kContract && m.h.nb == 4) return block_launch<kContract, 4, 4>(m, rho, vals, st);
     if (m.d.bsrc == kContract) return block_launch<kContract, 8, 2>(m, rho, vals, st);
     if (m.d.bsrc == kUniform) return block_launch<kUniform, 8, 2>(m, rho, vals, st);
     return block_launch<kStream, 8, 2>(m, rho, vals, st);
