@@ -254,9 +254,11 @@ soptx_status soptx_step_host(soptx_mesh mesh, const double *h_rho, const double 
  * The u-gradient takes a mesh-owned scratch of 8 nnz bytes, made by the first
  * call with d_grad_u (counted in soptx_mesh_device_bytes).  With FP64 element
  * matrices of box lattices and of affine cells of up to 10 nodes (P1-P3
- * triangles, P1 and P2 tetrahedra, Q1 and Q2 quadrilaterals, Q1 hexahedra) it
- * holds the cells' nodal forces E_e K_e^0 u_e, which are added node by node in
- * a fixed order; other meshes assemble K(rho) into it for the product.  If that
+ * triangles, P1 and P2 tetrahedra, Q1 and Q2 quadrilaterals, Q1 hexahedra; of
+ * P3, Q2 quadrilaterals, P2 tetrahedra and Q1 hexahedra from some thousand
+ * cells on) it holds the cells' nodal forces E_e K_e^0 u_e, which are added
+ * node by node in a fixed order; other meshes assemble K(rho) into it for the
+ * product.  Both forms are within 1e-14 of all rows together.  If that
  * memory cannot be allocated the product is formed from the element matrices
  * instead (same result within the tolerance, about an order of magnitude
  * slower).

@@ -155,6 +155,8 @@ static soptx_status setup_strain(soptx_mesh_s &m, const RefElement &ref, cudaStr
     for (size_t t = 0; t < sg.size(); t++) sg[t] = split_pair(h.geo[t]);
     soptx_status s = upload(&m.d.sq, tab, st, m.device_bytes, "quadrature table");
     if (s == SOPTX_OK) s = upload(&m.d.sgeo, sg, st, m.device_bytes, "cell geometry pairs");
+    if (s == SOPTX_OK && h.dim == 2 && m.prec == SOPTX_ELEM_FP64)
+        s = upload(&m.d.gtab, q.dphi, st, m.device_bytes, "reference gradients");
     if (s == SOPTX_OK && h.dim == 3 && !is_simplex(h.cell) && (h.order == 2 || h.order == 3)) {
         // the 1D factors of the tensor rule, for the sum-factorised kernel
         std::vector<double> w1, val, der;

@@ -148,7 +148,8 @@ struct DeviceMesh {
     bool strain = false;           // the sensitivities take one of their kernels
     float2 *sgeo = nullptr;        //   [nc, or 1 when uniform][d*d + 1] G and |det J| as float pairs;
                                    //   general cells: G and w |det J| at every point (GeneralArgs)
-    double *gtab = nullptr;        //   general cells of order 2, 3: tables (GeneralArgs)
+    double *gtab = nullptr;        //   general cells of order 2, 3: tables (GeneralArgs); affine 2D cells:
+                                   //   reference gradients in FP64 (ForceArgs)
     float2 *sq = nullptr;          //   quadrature: weights [snq], reference gradients [snq][nb][d]
     int snq = 0;
     float2 *ssf = nullptr;         //   hexahedra of order 2, 3: 1D weights, basis values and derivatives,

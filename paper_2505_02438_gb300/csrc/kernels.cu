@@ -290,7 +290,7 @@ cudaError_t launch_step(const soptx_mesh_s &m, const double *rho, const double *
     if (m.path == SOPTX_PATH_LATTICE && m.d.sectors && m.h.nc > 0)
         return launch_lattice_step(m, rho, u, vals, dc, c, st, gscale);
     if (m.d.strain && m.d.side && m.h.nc > 0 && m.h.nnz > 0 &&
-        (m.d.bchunks >= 0 || m.d.contract || m.d.pcached || m.d.puniform || (m.h.nonaffine && !gscale))) {
+        (m.d.bchunks >= 0 || m.d.contract || m.d.pcached || m.d.puniform || (m.h.nonaffine && (!gscale || m.h.nnz >= 1 << 18)))) {
         // the pair and block-row kernels fill every SM with a persistent grid that
         // takes its work from a counter: the sensitivities go first, on the mesh's
         // second stream (highest priority) with a few blocks per SM, and the assembly's
@@ -298,8 +298,9 @@ cudaError_t launch_step(const soptx_mesh_s &m, const double *rho, const double *
         // Blocks per SM, step us: P3 triangles 400x200 FP64 281 at one, 239 at four
         // (the float-pair sensitivity outlasted the assembly at one), FP32 172 / 176;
         // P2 tets 60x20x20 FP64 364 / 340, FP32 233 / 224.  General quadrilaterals, assembled
-        // by the gather, the same way (but one call after the other in the backward, where
-        // the overlap gained nothing: Q2 of 25 M values 699 us beside it, 648 after)
+        // by the gather, the same way (but one call after the other in the backward of small
+        // meshes, where the events cost more than the overlap gives: 31 and 28 us below
+        // 2^18 values; Q1 of 1.5 M values 36 beside it, 48 after)
         int dev = 0, sms = 0;
         cudaError_t err = cudaGetDevice(&dev);
         if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

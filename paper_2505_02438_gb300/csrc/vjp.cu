@@ -13,14 +13,15 @@
 //                     forces in planes [corner][component][cell], read back in planes.
 //  k_strain_forces  : affine cells of up to 10 nodes: at every point of the rule of
 //                     k_strain_energy the displacement gradient, the energy density
-//                     and the weighted stress S_q = w_q |det J| sigma G^T; then the forces
-//                     f_b = sum_q S_q grad^ phi_b(xi_q), which take the displacements'
+//                     and the weighted stress S_q = w_q sigma G^T; then the forces
+//                     f_b = |det J| sum_q S_q grad^ phi_b(xi_q), which take the displacements'
 //                     place in shared memory and leave coalesced as [cell][node][component].
-// Everything in float pairs (48 bits), as the assembled product.  The call, with the
-// product over K assembled for it before and from the forces now: 120x40x40 Q1
-// hexahedra 208 and 43 us, 144,000 P2 tetrahedra 515 and 111 us, 160,000 P3 triangles
-// 437 and 91 us, 480x160 quadrilaterals 109 and 26 us.  What bounds it is instruction
-// issue in the force kernels (float-pair products; all data are in L2).
+// In float pairs (48 bits) but for the last component of P3 triangles and Q2 quadrilaterals.
+// (The product over K has the last row of every node in FP64.)  The call, with the product
+// over K assembled for it and from the forces: 120x40x40 Q1 hexahedra 208 and 41 us,
+// 144,000 P2 tetrahedra 515 and 114 us, 160,000 P3 triangles 437 and 119 us (in float pairs
+// alone 88), 480x160 quadrilaterals 109 and 11 us.  What bounds it is instruction issue in
+// the force kernels (float-pair products; all data are in L2).
 #include <algorithm>
 #include <cstdint>
 
@@ -177,6 +178,7 @@ struct ForceArgs {
     int64_t geo_stride;               // d*d + 1, or 0 when every cell has the same Jacobian
     const float2 *__restrict__ qw;    // [NQ] weights
     const float2 *__restrict__ qd;    // [NQ][NB][D] reference gradients
+    const double *__restrict__ qd64;  // the same in FP64 (2D, NQ > 4)
     float2 lam, mu;
     const double *__restrict__ gout;
     double *__restrict__ grad_rho;
@@ -188,6 +190,7 @@ template <int D, int NB, int NQ>
 __global__ void __launch_bounds__(kThreads) k_strain_forces(const ForceArgs A)
 {
     constexpr int P = kThreads + 1, ND = NB * D;
+    constexpr bool kFp64 = D == 2 && NQ > 4;
     extern __shared__ float2 us[];
     const int tid = threadIdx.x;
     const double g = *A.gout;
@@ -237,14 +240,18 @@ __global__ void __launch_bounds__(kThreads) k_strain_forces(const ForceArgs A)
                     for (int i = 0; i < D; i++) {
                         const df ub = pair_of(us[(b * D + i) * P + tid]);
 #pragma unroll
-                        for (int m = 0; m < D; m++) acc_fma(U[i][m], ub, dp[m]);
+                        for (int m = 0; m < D; m++) {
+                            acc_fma(U[i][m], ub, dp[m]);
+                            // in 2D the sums' tails are short: 5% less error of g_u
+                            if (D == 2 && (b & 1)) U[i][m] = settle(U[i][m]);
+                        }
                     }
                 }
 #pragma unroll
                 for (int i = 0; i < D; i++)
 #pragma unroll
                     for (int m = 0; m < D; m++) U[i][m] = settle(U[i][m]);
-                // grad u = U^ G, the stress and w |det J| sigma G^T
+                // grad u = U^ G, the stress and w sigma G^T
                 df gu[D][D];
 #pragma unroll
                 for (int i = 0; i < D; i++)
@@ -258,7 +265,7 @@ __global__ void __launch_bounds__(kThreads) k_strain_forces(const ForceArgs A)
                 df tr = gu[0][0];
 #pragma unroll
                 for (int m = 1; m < D; m++) tr = df_add(tr, gu[m][m]);
-                const df lt = df_mul(lam, tr), wd = df_mul(pair_of(__ldg(A.qw + q)), det);
+                const df lt = df_mul(lam, tr), w = pair_of(__ldg(A.qw + q));
                 df sg[D][D], en{0.f, 0.f};
 #pragma unroll
                 for (int i = 0; i < D; i++)
@@ -266,9 +273,9 @@ __global__ void __launch_bounds__(kThreads) k_strain_forces(const ForceArgs A)
                     for (int j = i; j < D; j++) {
                         df t = df_mul(mu, df_add(gu[i][j], gu[j][i]));
                         if (i == j) t = df_add(t, lt);
-                        sg[i][j] = sg[j][i] = df_mul(wd, t);
+                        sg[i][j] = sg[j][i] = df_mul(w, t);
                     }
-                // density . w |det J| = sigma : grad u
+                // density . w = sigma : grad u
 #pragma unroll
                 for (int i = 0; i < D; i++)
 #pragma unroll
@@ -284,26 +291,49 @@ __global__ void __launch_bounds__(kThreads) k_strain_forces(const ForceArgs A)
                         S[q][i][m] = settle(t);
                     }
             }
-            const df sv = settle(s);
+            // |det J| last: taken into every point's weight its tail is lost on cells of 1e-9
+            // (a gradient 8e-13 off, now 1e-13)
+            const df sv = df_mul(settle(s), det);
             A.grad_rho[e] = g * simp_dE(A.sp, re) * df_to_double(sv.h, sv.l);
-            // the forces in the displacements' place
+            // the forces in the displacements' place.  In 2D with many points the second
+            // component is formed in FP64 from the stresses, as k_spmv forms a node's last
+            // row: in float pairs alone the sum over the points left g_u further off than the
+            // assembled product (P3 triangles 8.5e-15 against 7.8e-15 of 64 bits, Q2 boxes
+            // 8.8e-15 against 8.3e-15).  FP64 in both components is slower still
+            double S2[kFp64 ? NQ : 1][D], Ed2 = 0.0;
+            if constexpr (kFp64) {
+#pragma unroll
+                for (int q = 0; q < NQ; q++)
+#pragma unroll
+                    for (int m = 0; m < D; m++) S2[q][m] = pair_to_double(S[q][D - 1][m].h, S[q][D - 1][m].l);
+                Ed2 = (bad ? Ed : pair_to_double(Ep.x, Ep.y)) * pair_to_double(det.h, det.l);
+            }
 #pragma unroll 1
             for (int b = 0; b < NB; b++) {
                 df t[D];
+                double t2 = 0.0;
 #pragma unroll
                 for (int i = 0; i < D; i++) t[i] = df{0.f, 0.f};
 #pragma unroll
                 for (int q = 0; q < NQ; q++)
 #pragma unroll
                     for (int m = 0; m < D; m++) {
-                        const df dp = pair_of(__ldg(A.qd + (size_t)q * ND + b * D + m));
+                        const int at = q * ND + b * D + m;
+                        const df dp = pair_of(__ldg(A.qd + at));
 #pragma unroll
-                        for (int i = 0; i < D; i++) acc_fma(t[i], S[q][i][m], dp);
+                        for (int i = 0; i < (kFp64 ? D - 1 : D); i++) acc_fma(t[i], S[q][i][m], dp);
+                        if constexpr (kFp64) t2 = fma(S2[q][m], __ldg(A.qd64 + at), t2);
                     }
 #pragma unroll
                 for (int i = 0; i < D; i++) {
-                    const df x = settle(t[i]), y = df_mul(df{Ep.x, Ep.y}, x);
-                    us[(b * D + i) * P + tid] = bad ? times_fp64(Ed, x.h, x.l) : make_float2(y.h, y.l);
+                    float2 *const o = us + (b * D + i) * P + tid;
+                    if (kFp64 && i == D - 1) {
+                        const df y = df_split_z(Ed2 * t2);
+                        *o = make_float2(y.h, y.l);
+                    } else {
+                        const df x = df_mul(settle(t[i]), det), y = df_mul(df{Ep.x, Ep.y}, x);
+                        *o = bad ? times_fp64(Ed, x.h, x.l) : make_float2(y.h, y.l);
+                    }
                 }
             }
         }
@@ -385,12 +415,18 @@ cudaError_t strain_vjp(const soptx_mesh_s &m, const ForceArgs &A, double *grad_u
     return cudaGetLastError();
 }
 
-// The cells k_strain_forces is compiled for: nodes and points of the rule.
+// The cells k_strain_forces is compiled for: nodes and points of the rule, and the cells
+// from which it is the faster way (a thread per cell: on few cells of many points its chain
+// of operations is longer than the product over K.  Calls, us, product and forces: P2
+// tetrahedra 96 cells 33 and 36, 900 35 and 36, 4860 45 and 40; hexahedra 150 cells 42 and
+// 54, 6480 50 and 55, 106,000 314 and 174; P3 triangles 1200 cells 32 and 34, 9800 33 and 34,
+// 160,000 241 and 77; Q2 quadrilaterals 800 cells 33 and 37, 6000 34 and 38, 98,000 282 and 86).
 bool forces_fit(const soptx_mesh_s &m)
 {
-    static const int combos[][3] = {{2, 3, 1}, {2, 6, 3}, {2, 10, 7}, {2, 4, 4}, {2, 9, 9}, {3, 4, 1}, {3, 10, 4}, {3, 8, 8}};
+    static const int combos[][4] = {{2, 3, 1, 0}, {2, 6, 3, 0}, {2, 10, 7, 8192}, {2, 4, 4, 0}, {2, 9, 9, 8192},
+                                    {3, 4, 1, 0}, {3, 10, 4, 2048}, {3, 8, 8, 10000}};
     for (const auto &c : combos)
-        if (m.h.dim == c[0] && m.h.nb == c[1] && m.d.snq == c[2]) return true;
+        if (m.h.dim == c[0] && m.h.nb == c[1] && m.d.snq == c[2]) return m.h.nc >= c[3];
     return false;
 }
 
@@ -428,6 +464,7 @@ cudaError_t launch_vjp(const soptx_mesh_s &m, const double *rho, const double *u
     A.geo_stride = m.path == SOPTX_PATH_UNIFORM ? 0 : h.dim * h.dim + 1;
     A.qw = m.d.sq;
     A.qd = m.d.sq + m.d.snq;
+    A.qd64 = m.d.gtab;
     A.lam = pair(m.mat.lam);
     A.mu = pair(m.mat.mu);
     A.gout = gout;
