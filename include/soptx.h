@@ -413,6 +413,14 @@ soptx_status soptx_measure_pipe_rates(soptx_pipe_rates *out);
  * (n >= 1) fails as if the device were out of memory; n <= 0 disables. */
 void soptx_debug_fail_alloc_after(int64_t n);
 
+/* Test hook: the limit of the waits inside the assembly kernel of this mesh, in
+ * tries (0: every wait runs out at once; negative: the library's own limit of
+ * about a second).  When a wait runs out the kernel leaves with K incomplete;
+ * the next call on the mesh (a solve: the same call) returns SOPTX_ECUDA, once,
+ * and a served request its own result.  Only 3D meshes off the box lattice have
+ * such waits. */
+void soptx_debug_mesh_wait_tries(soptx_mesh mesh, int32_t tries);
+
 /* Test hook for the lattice path: while enabled (nonzero), meshes created
  * from now on skip the Walsh-sector split of the box element, so their
  * sensitivities take the general gather kernels (the route a box whose

@@ -115,6 +115,7 @@ SIGNATURES = {
     "soptx_measure_pipe_rates": (i32, [ctypes.POINTER(PipeRates)]),
     "soptx_debug_fail_alloc_after": (None, [i64]),
     "soptx_debug_lattice_no_sectors": (None, [i32]),
+    "soptx_debug_mesh_wait_tries": (None, [P, i32]),
 }
 
 _lib = None

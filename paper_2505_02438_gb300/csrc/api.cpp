@@ -40,6 +40,7 @@ static void free_device(DeviceMesh &d)
                     d.bblob, d.bcoff, d.bcell, d.bM, d.bkblk, d.cticket, d.rbuf};
     for (void *p : ptrs)
         if (p) cudaFree(p);
+    if (d.bexpired) cudaFreeHost((void *)d.bexpired);
     if (d.cg_exec) cudaGraphExecDestroy(d.cg_exec);
     if (d.cg_cap) cudaStreamDestroy(d.cg_cap);
     for (cudaEvent_t e : d.ev)
@@ -586,12 +587,17 @@ static soptx_status setup_block_rows(soptx_mesh_s &m, const RefElement &ref, con
         m.d.bblob = reinterpret_cast<uint4 *>(p);
     }
     if (s == SOPTX_OK) s = upload(&m.d.bcoff, T.coff, st, m.device_bytes, "chunk offsets");
-    if (s == SOPTX_OK) s = upload(&m.d.cticket, std::vector<unsigned>(4, 0u), st, m.device_bytes, "chunk counter");
+    if (s == SOPTX_OK) s = upload(&m.d.cticket, std::vector<unsigned>(2, 0u), st, m.device_bytes, "chunk counter");
+    if (s == SOPTX_OK) {
+        void *p = nullptr;
+        s = cuda_status(cudaHostAlloc(&p, 64, cudaHostAllocPortable | cudaHostAllocMapped), "error word");
+        m.d.bexpired = (volatile unsigned *)p;
+        if (s == SOPTX_OK) *m.d.bexpired = 0u;
+    }
     m.d.bcell_bits = T.cell_bits;
     m.d.bmax_blob = T.max_blob;
     m.d.bmax_cells = T.max_cells;
     m.d.bmax_stage = T.max_stage;
-    m.d.bmax_rows = T.max_rows;
     m.d.bsmem = (int)smem;
     m.d.bsrc = src;
     if (s == SOPTX_OK) m.d.bchunks = T.nchunks;
@@ -609,6 +615,13 @@ static soptx_status setup_block_rows(soptx_mesh_s &m, const RefElement &ref, con
     // (the host tables go out of scope: their copies have to be done)
     if (s == SOPTX_OK) s = cuda_status(cudaStreamSynchronize(st), "chunk records");
     return s;
+}
+
+soptx_status take_expired(const soptx_mesh_s &m)
+{
+    if (!m.d.bexpired || *m.d.bexpired == 0u) return SOPTX_OK;
+    *m.d.bexpired = 0u;
+    SOPTX_FAIL(SOPTX_ECUDA, "a wait in an earlier assembly of this mesh ran out: that K is incomplete");
 }
 
 static bool material_ok(const soptx_material *m, int dim, Material &out, std::string &err)
@@ -643,6 +656,10 @@ extern "C" {
 const char *soptx_last_error(void) { return g_last_error.c_str(); }
 const char *soptx_version(void) { return "soptx-gb300 0.1 (sm_103a)"; }
 void soptx_debug_fail_alloc_after(int64_t n) { g_fail_after.store(n > 0 ? n : 0); }
+void soptx_debug_mesh_wait_tries(soptx_mesh m, int32_t tries)
+{
+    if (m) m->d.btries = tries >= 0 ? tries : kBlockWaitTries;
+}
 void soptx_debug_lattice_no_sectors(int32_t enable) { g_no_sectors.store(enable ? 1 : 0); }
 
 soptx_status soptx_mesh_create(int dim, soptx_cell cell, int order, int64_t n_vertices, const double *coords,
@@ -1050,6 +1067,7 @@ soptx_status soptx_assemble_K(soptx_mesh m, const double *d_rho, double *d_vals,
 {
     if (!m) SOPTX_FAIL(SOPTX_EINVAL, "mesh is NULL");
     if ((!d_rho && m->h.nc > 0) || (!d_vals && m->h.nnz > 0)) SOPTX_FAIL(SOPTX_EINVAL, "d_rho / d_vals is NULL");
+    if (const soptx_status s = take_expired(*m)) return s;
     return cuda_status(launch_assemble(*m, d_rho, d_vals, (cudaStream_t)stream), "soptx_assemble_K");
 }
 
@@ -1058,6 +1076,7 @@ soptx_status soptx_sensitivity(soptx_mesh m, const double *d_rho, const double *
 {
     if (!m) SOPTX_FAIL(SOPTX_EINVAL, "mesh is NULL");
     if (m->h.nc > 0 && (!d_rho || !d_u || !d_dc)) SOPTX_FAIL(SOPTX_EINVAL, "d_rho / d_u / d_dc is NULL");
+    if (const soptx_status s = take_expired(*m)) return s;
     return cuda_status(launch_sensitivity(*m, d_rho, d_u, d_dc, d_c, -1.0, nullptr, (cudaStream_t)stream),
                        "soptx_sensitivity");
 }
@@ -1068,6 +1087,7 @@ soptx_status soptx_assemble_and_sensitivity(soptx_mesh m, const double *d_rho, c
     if (!m) SOPTX_FAIL(SOPTX_EINVAL, "mesh is NULL");
     if ((!d_vals && m->h.nnz > 0) || (m->h.nc > 0 && (!d_rho || !d_u || !d_dc)))
         SOPTX_FAIL(SOPTX_EINVAL, "d_rho / d_u / d_vals / d_dc is NULL");
+    if (const soptx_status s = take_expired(*m)) return s;
     if (((m->path == SOPTX_PATH_LATTICE && m->h.dim == 2 && m->d.sectors) || m->d.strain) && m->h.nc > 0) {
         cudaError_t e = ensure_side(*m);
         if (e != cudaSuccess) return cuda_status(e, "soptx_assemble_and_sensitivity stream");
@@ -1121,6 +1141,7 @@ soptx_status soptx_step_host(soptx_mesh m, const double *h_rho, const double *h_
     const auto &h = m->h;
     if ((!d_vals && h.nnz > 0) || (h.nc > 0 && !h_dc) || (h.nc > 0 && !h_rho) || (h.ndof > 0 && !h_u))
         SOPTX_FAIL(SOPTX_EINVAL, "h_rho / h_u / d_vals / h_dc is NULL");
+    if (const soptx_status s = take_expired(*m)) return s;
     auto &d = m->d;
     cudaError_t e = cudaSuccess;
     if (!d.stage) {
@@ -1182,6 +1203,7 @@ soptx_status soptx_compliance_vjp(soptx_mesh m, const double *d_rho, const doubl
     if (!d_gout) SOPTX_FAIL(SOPTX_EINVAL, "d_gout is NULL");
     if (m->h.nc > 0 && (!d_rho || !d_u || !d_grad_rho)) SOPTX_FAIL(SOPTX_EINVAL, "d_rho / d_u / d_grad_rho is NULL");
     if (d_grad_u && m->h.ndof > 0 && !d_u) SOPTX_FAIL(SOPTX_EINVAL, "d_u is NULL");
+    if (const soptx_status s = take_expired(*m)) return s;
     cudaStream_t st = (cudaStream_t)stream;
     auto &d = m->d;
     if (d_grad_u && !d.kvals && m->h.nnz > 0) {

@@ -76,10 +76,12 @@ constexpr int kRowBytes = 32 * 9 * 8;
 
 struct BlockArgs {
     int64_t nchunks;
-    unsigned *__restrict__ ticket;        // [0] chunks handed out, [1] CTAs done (both zero between calls), [2] error
+    unsigned *__restrict__ ticket;        // [0] chunks handed out, [1] CTAs done (both zero between calls)
+    volatile unsigned *expired;           // host memory: set when a wait ran out (the next call reports it)
+    int tries;                            // limit of a wait
     const uint4 *__restrict__ blob;
     const uint32_t *__restrict__ coff;    // [nchunks + 1] chunk starts in 16-byte units
-    int max_blob, max_cells, max_stage, max_rows, cell_bits;   // 16-byte units, cells, values, rows; of a record
+    int max_blob, max_cells, max_stage, cell_bits;   // 16-byte units, cells, values; of a record
     const float4 *__restrict__ cdata;     // kContract: [nc][3] G row-major, |det J|
     const float *__restrict__ M;          // kContract: reference integrals [nb nb][12]
     int nm;                               // floats in M
@@ -112,9 +114,10 @@ __device__ __forceinline__ void bulk_store(double *gdst, const double *ssrc, uin
                  : "memory");
 }
 
-// Shared-memory barriers (mbarrier).  Every wait is bounded: after kWaitTries
-// tries of up to 20 us each it gives up, the warp raises the error flag and leaves.
-constexpr int kWaitTries = 1 << 16;
+// Shared-memory barriers (mbarrier).  Every wait is bounded: after BlockArgs::tries tries
+// (kBlockWaitTries) of up to 20 us each the whole warp gives up, raises the error word and
+// leaves; the others' waits run out after it, and the data-moving warp still waits, with
+// the full limit, for the copies that it has in flight.
 __device__ __forceinline__ void mbar_init(uint64_t *b, unsigned count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(b)), "r"(count) : "memory");
@@ -123,9 +126,9 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *b)
 {
     asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_addr(b)) : "memory");
 }
-__device__ __forceinline__ bool mbar_wait(uint64_t *b, unsigned parity)
+__device__ __forceinline__ bool mbar_wait(uint64_t *b, unsigned parity, int tries)
 {
-    for (int i = 0; i < kWaitTries; i++) {
+    for (int i = 0; i < tries; i++) {
         unsigned done;
         asm volatile(
             "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 20000;\n\tselp.u32 %0, 1, 0, "
@@ -133,7 +136,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *b, unsigned parity)
             : "=r"(done)
             : "r"(smem_addr(b)), "r"(parity)
             : "memory");
-        if (done) return true;
+        if (__all_sync(kFull, (int)done)) return true;   // (the lanes decide alike)
     }
     return false;
 }
@@ -252,12 +255,11 @@ struct Blocks {
 
 // W warps assemble, one more moves data.  In step k that warp waits until the others
 // have left chunk k - 2 and hands its rows to the copy engine, starts the copy of
-// chunk k's streamed blocks and of record k + 2 into the places that chunk k - 2 had,
+// record k + 2 into the place that chunk k - 2 had,
 // gathers the cells of chunk k + 1 and opens it, and frees the place of chunk
 // k's rows once the copy engine has read the rows staged there.  The assembling warps
-// look for the streamed blocks when they enter a chunk, for the freed place only
-// before their first rows of it.  They are never more than two chunks
-// apart (chunk k + 2 opens once all have left chunk k - 1).
+// look for the freed place only before their first rows of a chunk.  They are never
+// more than two chunks apart (chunk k + 2 opens once all have left chunk k - 1).
 template <int SRC, int W, int MINB>
 __global__ void __launch_bounds__(32 * (W + 1), MINB) k_block_rows(const BlockArgs A)
 {
@@ -286,6 +288,12 @@ __global__ void __launch_bounds__(32 * (W + 1), MINB) k_block_rows(const BlockAr
     }
     __syncthreads();
 
+    auto raise = [&]() {
+        if (lane == 0) {
+            *A.expired = 1u;
+            __threadfence_system();
+        }
+    };
     if (warp == W) {
         const bool al16 = (reinterpret_cast<uintptr_t>(A.vals) & 15u) == 0;
         auto grab = [&]() -> int64_t {
@@ -300,8 +308,16 @@ __global__ void __launch_bounds__(32 * (W + 1), MINB) k_block_rows(const BlockAr
                 u1 = __ldg(A.coff + c + 1);
             }
         };
-        auto load_record = [&](uint32_t u0, uint32_t u1, int q) {
-            if (lane == 0 && u1 > u0) bulk_load(blobs + q * A.max_blob, A.blob + u0, 16u * (u1 - u0), &s_rec[q]);
+        int issued = 0, landed = 0;   // records on their way, and waited for: record i in place i mod 4
+        auto load_record = [&](uint32_t u0, uint32_t u1) {
+            if (u1 <= u0) return;
+            const int q = issued++ & 3;
+            if (lane == 0) bulk_load(blobs + q * A.max_blob, A.blob + u0, 16u * (u1 - u0), &s_rec[q]);
+        };
+        auto wait_record = [&](int tries) {
+            if (!mbar_wait(&s_rec[landed & 3], (landed >> 2) & 1, tries)) return false;
+            landed++;
+            return true;
         };
         auto record = [&](int k) { return reinterpret_cast<const uint32_t *>(blobs + (k & 3) * A.max_blob); };
         // the staged rows of the chunk with record B to the CSR values
@@ -359,16 +375,16 @@ __global__ void __launch_bounds__(32 * (W + 1), MINB) k_block_rows(const BlockAr
         uint32_t u0, u1;
         int64_t c = grab();
         bounds(c, u0, u1);
-        load_record(u0, u1, 0);
+        load_record(u0, u1);
         bool more = c < A.nchunks, ok = true;
         c = grab();
         bounds(c, u0, u1);
-        load_record(u0, u1, 1);
+        load_record(u0, u1);
         bool more1 = c < A.nchunks;   // chunk k + 1 exists
         c = grab();
         bounds(c, u0, u1);            // chunk k + 2
         if (more) {
-            ok = mbar_wait(&s_rec[0], 0);
+            ok = wait_record(A.tries);
             if (ok) gather_cells(record(0), cbuf);
             cp_async_wait_all();
         }
@@ -378,15 +394,15 @@ __global__ void __launch_bounds__(32 * (W + 1), MINB) k_block_rows(const BlockAr
             const int s = k & 1;
             q = q == 2 ? 0 : q + 1;
             if (k >= 2) {
-                ok = mbar_wait(&s_done[(k - 2) & 3], ((k - 2) >> 2) & 1);
+                ok = mbar_wait(&s_done[(k - 2) & 3], ((k - 2) >> 2) & 1, A.tries);
                 if (!ok) break;
                 store_rows(record(k - 2), stages + s * sstride);
             }
             if (!more) continue;
-            load_record(u0, u1, (k + 2) & 3);
+            load_record(u0, u1);
             const bool more2 = c < A.nchunks;
             if (more1) {
-                ok = mbar_wait(&s_rec[(k + 1) & 3], ((k + 1) >> 2) & 1);
+                ok = wait_record(A.tries);
                 if (!ok) break;
                 gather_cells(record(k + 1), cbuf + q * cstride);
                 last++;
@@ -402,7 +418,11 @@ __global__ void __launch_bounds__(32 * (W + 1), MINB) k_block_rows(const BlockAr
             more = more1;
             more1 = more2;
         }
-        if (!ok && lane == 0) atomicExch(A.ticket + 2, 1u);
+        if (!ok) {
+            raise();
+            while (landed < issued && wait_record(kBlockWaitTries)) {
+            }
+        }
         cp_async_wait_all();
         asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
         // the last CTA to finish sets the counter back to zero for the next call
@@ -418,14 +438,11 @@ __global__ void __launch_bounds__(32 * (W + 1), MINB) k_block_rows(const BlockAr
     }
 
     const uint32_t cmask = (1u << A.cell_bits) - 1u;
-    auto give_up = [&]() {
-        if (lane == 0) atomicExch(A.ticket + 2, 1u);
-    };
     int q = 0;
     unsigned pq = 0;   // parity of s_full[q]
     for (int k = 0;; k++) {
         const int s = k & 1;
-        if (!mbar_wait(&s_full[q], pq)) return give_up();
+        if (!mbar_wait(&s_full[q], pq, A.tries)) return raise();
         if (!s_more[q]) return;
         const uint32_t *B = reinterpret_cast<const uint32_t *>(blobs + (k & 3) * A.max_blob);
         const unsigned char *const cb = cbuf + q * cstride;
@@ -519,7 +536,7 @@ __global__ void __launch_bounds__(32 * (W + 1), MINB) k_block_rows(const BlockAr
             for (int p = 0; p < 9; p++) big = max_nan(big, fabsf(v[p].x));
             bad |= !(big <= FLT_MAX);
             if (!free) {
-                if (!mbar_wait(&s_free[s], (k >> 1) & 1)) return give_up();
+                if (!mbar_wait(&s_free[s], (k >> 1) & 1, A.tries)) return raise();
                 free = true;
             }
             const uint32_t o1 = pr.x & 0xffffu;
@@ -602,12 +619,13 @@ cudaError_t block_launch(const soptx_mesh_s &m, const double *rho, double *vals,
     BlockArgs A;
     A.nchunks = d.bchunks;
     A.ticket = d.cticket;
+    A.expired = d.bexpired;
+    A.tries = d.btries;
     A.blob = d.bblob;
     A.coff = d.bcoff;
     A.max_blob = d.bmax_blob;
     A.max_cells = d.bmax_cells;
     A.max_stage = d.bmax_stage;
-    A.max_rows = d.bmax_rows;
     A.cell_bits = d.bcell_bits;
     A.cdata = d.bcell;
     A.M = d.bM;
@@ -640,7 +658,7 @@ cudaError_t block_launch(const soptx_mesh_s &m, const double *rho, double *vals,
 int64_t block_row_bytes() { return kRowBytes; }
 
 // Shared memory of a CTA: two chunks' staged rows, four chunk records, three chunks' cells,
-// then the reference integrals or two chunks' streamed blocks.
+// then the reference integrals (kContract).
 int64_t block_smem(int src, int nb, const BlockTables &T)
 {
     const int64_t cb = src == kContract ? kCellBytes<kContract> : kCellBytes<kUniform>;

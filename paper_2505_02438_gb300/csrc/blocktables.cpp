@@ -278,7 +278,6 @@ bool build_chunks(const HostMesh &h, const BlockLimits &L, const std::vector<int
             place++;
         }
         B[b0 + 1] |= row << 16;
-        T.max_rows = std::max(T.max_rows, (int)row);
         T.rows += row;
         B.resize((B.size() + 3) & ~(size_t)3, 0u);
         T.max_blob = std::max(T.max_blob, (int)((B.size() - b0) / 4));
@@ -373,7 +372,6 @@ bool build_block_tables(const HostMesh &h, const double *coords, const int32_t *
         T.blob.insert(T.blob.end(), P.blob.begin(), P.blob.end());
         std::vector<uint32_t>().swap(P.blob);
         T.rows += P.rows;
-        T.max_rows = std::max(T.max_rows, P.max_rows);
         T.max_blob = std::max(T.max_blob, P.max_blob);
         T.max_cells = std::max(T.max_cells, P.max_cells);
         T.max_stage = std::max(T.max_stage, P.max_stage);

@@ -92,6 +92,7 @@ void build_csr(const HostMesh &hm, std::vector<int64_t> &indptr, std::vector<int
 // ---------------------------------------------------------------- block rows
 // Tables of the block-row kernel of 3D meshes (blockrows.cu, where the layout is described).
 constexpr int kBlockHead = 5;   // words before a record's nodes
+constexpr int kBlockWaitTries = 1 << 16;   // limit of the kernel's waits, about a second
 struct BlockLimits {
     int blocks = 432;    // row blocks of a chunk (a larger node is a chunk of its own)
     int cells = 110;     // cells of a chunk
@@ -105,7 +106,6 @@ struct BlockTables {
     std::vector<uint32_t> coff;   // [nchunks + 1] their starts in 16-byte units
     int64_t nchunks = 0, rows = 0;
     int cell_bits = 0;            // bits of a record that name the chunk's cell
-    int max_rows = 0;             // most record rows of a chunk
     int max_blob = 0;             // largest record in 16-byte units
     int max_cells = 0, max_stage = 0, max_nodes = 0;   // most cells, staged values and nodes of a chunk
 };
@@ -172,14 +172,16 @@ struct DeviceMesh {
     int64_t bchunks = -1;          //   chunks (-1: the mesh's assembly is another kernel's)
     int bsmem = 0;                 //   shared memory of a CTA
     int bsrc = 0;                  //   where the blocks come from (kBlockContract, ...)
-    int bmax_blob = 0, bmax_cells = 0, bmax_stage = 0, bmax_rows = 0, bcell_bits = 0;   // see BlockTables
+    int bmax_blob = 0, bmax_cells = 0, bmax_stage = 0, bcell_bits = 0;   // see BlockTables
     uint4 *bblob = nullptr;        //   chunk records
     uint32_t *bcoff = nullptr;     //   [bchunks + 1] their starts
     float4 *bcell = nullptr;       //   kBlockContract: [nc][3] G, |det J| in FP32
     float *bM = nullptr;           //   kBlockContract: reference integrals [nb][nb][12] in FP32
     float4 *bkblk = nullptr;       //   kBlockUniform: the blocks of the one element matrix
                                    //   kBlockStream: every record's block, in the kernel's order
-    unsigned *cticket = nullptr;   // [4] chunk counter, finished CTAs (both zero between calls), error flag
+    unsigned *cticket = nullptr;   // [2] chunk counter, finished CTAs (both zero between calls)
+    volatile unsigned *bexpired = nullptr;   // block rows: a word of pinned host memory, set by a wait that ran out
+    int btries = kBlockWaitTries;  //   limit of its waits
     // equilibrium solve (allocated by the first soptx_solve_cg)
     double *cg = nullptr;          // r z p q diag [ndof], scalars, partials, counters
     cudaGraphExec_t cg_exec = nullptr; // the CG iterations between two checks, as a graph
@@ -269,6 +271,8 @@ int64_t block_row_bytes();   // a record row of streamed blocks
 int64_t block_smem(int src, int nb, const BlockTables &T);
 cudaError_t launch_block_stream(const soptx_mesh_s &m, cudaStream_t st);
 cudaError_t launch_block_rows(const soptx_mesh_s &m, const double *rho, double *vals, cudaStream_t st);
+// ECUDA, once, after an assembly of this mesh whose waits ran out (its K is incomplete); no synchronisation
+soptx_status take_expired(const soptx_mesh_s &m);
 // contract.cu
 bool contract_fits(int dim, int nb, int max_deg);
 bool pairs_fit(int dim, int nb, int max_deg);

@@ -168,7 +168,9 @@ struct soptx_server_s {
             q->res.gpu_start_us = 1e3 * ms0;
             q->res.gpu_end_us = 1e3 * ms1;
             q->job->in_flight--;
-            finish(q, e == cudaSuccess ? SOPTX_OK : SOPTX_ECUDA);
+            soptx_status st = e == cudaSuccess ? SOPTX_OK : SOPTX_ECUDA;
+            if (st == SOPTX_OK && q->job->mesh) st = soptx::take_expired(*q->job->mesh);
+            finish(q, st);
             inflight.erase(inflight.begin() + k);
         }
     }

@@ -386,6 +386,7 @@ soptx_status soptx_spmv(soptx_mesh m, const double *d_vals, const double *d_x, d
 {
     if (!m) SOPTX_FAIL(SOPTX_EINVAL, "mesh is NULL");
     if (m->h.nnz > 0 && (!d_vals || !d_x || !d_y)) SOPTX_FAIL(SOPTX_EINVAL, "d_vals / d_x / d_y is NULL");
+    if (const soptx_status s = take_expired(*m)) return s;
     return cuda_fail(launch_spmv(*m, d_vals, d_x, d_y, nullptr, nullptr, nullptr, nullptr, nullptr,
                                  (cudaStream_t)stream),
                      "soptx_spmv");
@@ -440,6 +441,8 @@ soptx_status soptx_solve_cg(soptx_mesh m, const double *d_vals, const uint8_t *d
     if (e == cudaSuccess) e = cudaMemcpyAsync(&bad_h, bad, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "soptx_solve_cg");
+    // (the stream has been waited for: an assembly before this call is over)
+    if (const soptx_status s = take_expired(*m)) return s;
     if (bad_h) SOPTX_FAIL(SOPTX_EINVAL, "a free dof has a non-positive diagonal (no element touches it?)");
 
     // the scale of the residual test: ||f - K u_D|| on the free rows
