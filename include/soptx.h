@@ -108,6 +108,12 @@ typedef enum {
  * Allocates device memory (reported by soptx_mesh_device_bytes) and
  * synchronises `stream`.  Errors: EINVAL (bad sizes, ids, a degenerate or
  * inverted cell, ndof >= 2^31), ENOMEM, ECUDA.  n_cells = 0 is allowed.
+ * Cells of differing shapes hold their element matrices (8 or 4 ldof^2 bytes a
+ * cell).  3D meshes with FP64 ones hold the blocks a second time in the order
+ * of the assembly, 1.7 to 1.9 times the bytes without; general (bilinear,
+ * trilinear) cells with FP64 ones 8 (dim^2 + 1) bytes per Gauss point.  Where
+ * these cannot be had the mesh is made without them and served by the row
+ * gather (soptx_mesh_routes).
  */
 soptx_status soptx_mesh_create(int dim, soptx_cell cell, int order,
                                int64_t n_vertices, const double *coords,
@@ -153,7 +159,8 @@ soptx_status soptx_mesh_path(soptx_mesh mesh, soptx_path *path);
  *                  order (k_block_rows)
  *   *sensitivity : 0 box lattice (Walsh sectors), 1 fused into the row
  *                  gather, 2 strain energy at quadrature points
- *                  (k_strain_energy: affine cells)
+ *                  (k_strain_energy: affine cells; k_strain_corners and
+ *                  k_strain_tensor: general ones with FP64 element matrices)
  * Either pointer may be NULL.
  */
 soptx_status soptx_mesh_routes(soptx_mesh mesh, int32_t *assembly, int32_t *sensitivity);

@@ -4,6 +4,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <initializer_list>
 #include <new>
 
 #include "internal.h"
@@ -100,6 +101,18 @@ static soptx_status upload(T **dst, const std::vector<T> &src, cudaStream_t st, 
     return SOPTX_OK;
 }
 
+// Frees device arrays and takes them off the mesh's count again.
+static void drop_arrays(soptx_mesh_s &m, std::initializer_list<void **> arrays, int64_t bytes_before)
+{
+    for (void **a : arrays) {
+        if (*a) cudaFree(*a);
+        *a = nullptr;
+    }
+    m.device_bytes = bytes_before;
+    cudaGetLastError();
+    set_error("");
+}
+
 static float2 split_pair(double x)
 {
     const float hh = (float)x;
@@ -108,7 +121,7 @@ static float2 split_pair(double x)
 
 // General cells (strain_general.cu): the geometry of every Gauss point, computed on the
 // device, and the tables of orders 2 and 3.
-static soptx_status setup_strain_general(soptx_mesh_s &m, const RefElement &ref, cudaStream_t st)
+static soptx_status build_strain_general(soptx_mesh_s &m, const RefElement &ref, cudaStream_t st)
 {
     const HostMesh &h = m.h;
     std::vector<double> tab;
@@ -137,6 +150,17 @@ static soptx_status setup_strain_general(soptx_mesh_s &m, const RefElement &ref,
     }
     m.device_bytes += (int64_t)bytes;
     m.d.strain = true;
+    return SOPTX_OK;
+}
+
+// The same, leaving the sensitivities to the gather when the memory cannot be had.
+static soptx_status setup_strain_general(soptx_mesh_s &m, const RefElement &ref, cudaStream_t st)
+{
+    const int64_t before = m.device_bytes;
+    const soptx_status s = build_strain_general(m, ref, st);
+    if (s != SOPTX_ENOMEM) return s;
+    cudaStreamSynchronize(st);
+    drop_arrays(m, {(void **)&m.d.gtab, (void **)&m.d.sgeo}, before);
     return SOPTX_OK;
 }
 
@@ -521,7 +545,7 @@ static bool build_row_tables(const HostMesh &h, RowTables &T)
 
 // Tables of the block-row kernel of 3D meshes (blockrows.cu).  The mesh keeps the
 // cached gather when its largest node does not fit in the tables or in shared memory.
-static soptx_status setup_block_rows(soptx_mesh_s &m, const RefElement &ref, const double *coords, const int32_t *cv,
+static soptx_status build_block_rows(soptx_mesh_s &m, const RefElement &ref, const double *coords, const int32_t *cv,
                                      int src, cudaStream_t st)
 {
     const HostMesh &h = m.h;
@@ -615,6 +639,30 @@ static soptx_status setup_block_rows(soptx_mesh_s &m, const RefElement &ref, con
     // (the host tables go out of scope: their copies have to be done)
     if (s == SOPTX_OK) s = cuda_status(cudaStreamSynchronize(st), "chunk records");
     return s;
+}
+
+// The same, keeping the gather as well when the memory cannot be had: with the cached FP64
+// matrices the tables and the streamed blocks nearly double a mesh, and the gather needs
+// neither.
+static soptx_status setup_block_rows(soptx_mesh_s &m, const RefElement &ref, const double *coords, const int32_t *cv,
+                                     int src, cudaStream_t st)
+{
+    auto &d = m.d;
+    const int64_t before = m.device_bytes;
+    soptx_status s;
+    try {
+        s = build_block_rows(m, ref, coords, cv, src, st);
+    } catch (const std::bad_alloc &) {
+        s = SOPTX_ENOMEM;
+    }
+    if (s != SOPTX_ENOMEM) return s;
+    cudaStreamSynchronize(st);
+    drop_arrays(m, {(void **)&d.bblob, (void **)&d.bcoff, (void **)&d.bcell, (void **)&d.bM, (void **)&d.bkblk, (void **)&d.cticket},
+                before);
+    if (d.bexpired) cudaFreeHost((void *)d.bexpired);
+    d.bexpired = nullptr;
+    d.bchunks = -1;
+    return SOPTX_OK;
 }
 
 soptx_status take_expired(const soptx_mesh_s &m)
@@ -813,6 +861,21 @@ soptx_status soptx_mesh_create(int dim, soptx_cell cell, int order, int64_t n_ve
         }
         if (s == SOPTX_OK) s = cuda_status(cudaStreamSynchronize(st), "mesh setup");
     }
+    if (s == SOPTX_OK && (m->path != SOPTX_PATH_LATTICE || !d.sectors)) {
+        // per-call float-pair moduli and displacements, per-(cell, node) partials
+        // of the general path (also the sensitivity of a lattice whose element
+        // matrix does not split into Walsh sectors); before the tables that a mesh can do without
+        void *p1 = nullptr, *p2 = nullptr, *p3 = nullptr;
+        cudaError_t e = d.Edf ? cudaSuccess : dev_alloc(&p1, (size_t)std::max<int64_t>(h.nc, 1) * sizeof(float2));
+        if (e == cudaSuccess) e = dev_alloc(&p2, (size_t)std::max<int64_t>(h.ndof, 1) * sizeof(float2));
+        if (e == cudaSuccess) e = dev_alloc(&p3, (size_t)std::max<int64_t>(h.nc * h.nb, 1) * sizeof(double));
+        if (!d.Edf) d.Edf = (float2 *)p1;
+        d.udf = (float2 *)p2;
+        d.part = (double *)p3;
+        if (e != cudaSuccess) { cudaGetLastError(); s = cuda_status(e, "general-path scratch"); }
+        else B += (p1 ? std::max<int64_t>(h.nc, 1) * 8 : 0) + std::max<int64_t>(h.ndof, 1) * 8 +
+                  std::max<int64_t>(h.nc * h.nb, 1) * 8;
+    }
     if (s == SOPTX_OK && m->path != SOPTX_PATH_LATTICE && h.nc > 0 && (!h.nonaffine || prec == SOPTX_ELEM_FP64)) {
         // affine cells off the lattice: the sensitivities from the strain energy at
         // the points of a rule exact for it (G and |det J| per cell as float pairs,
@@ -836,27 +899,7 @@ soptx_status soptx_mesh_create(int dim, soptx_cell cell, int order, int64_t n_ve
         const int src = m->path == SOPTX_PATH_UNIFORM                   ? kBlockUniform
                         : prec == SOPTX_ELEM_FP32          ? kBlockContract
                                                                   : kBlockStream;
-        try {
-            s = setup_block_rows(*m, ref, coords, cell_vertices, src, st);
-        } catch (const std::bad_alloc &) {
-            set_error("host allocation failed building the chunk records");
-            s = SOPTX_ENOMEM;
-        }
-    }
-    if (s == SOPTX_OK && (m->path != SOPTX_PATH_LATTICE || !d.sectors)) {
-        // per-call float-pair moduli and displacements, per-(cell, node) partials
-        // of the general path (also the sensitivity of a lattice whose element
-        // matrix does not split into Walsh sectors)
-        void *p1 = nullptr, *p2 = nullptr, *p3 = nullptr;
-        cudaError_t e = d.Edf ? cudaSuccess : dev_alloc(&p1, (size_t)std::max<int64_t>(h.nc, 1) * sizeof(float2));
-        if (e == cudaSuccess) e = dev_alloc(&p2, (size_t)std::max<int64_t>(h.ndof, 1) * sizeof(float2));
-        if (e == cudaSuccess) e = dev_alloc(&p3, (size_t)std::max<int64_t>(h.nc * h.nb, 1) * sizeof(double));
-        if (!d.Edf) d.Edf = (float2 *)p1;
-        d.udf = (float2 *)p2;
-        d.part = (double *)p3;
-        if (e != cudaSuccess) { cudaGetLastError(); s = cuda_status(e, "general-path scratch"); }
-        else B += (p1 ? std::max<int64_t>(h.nc, 1) * 8 : 0) + std::max<int64_t>(h.ndof, 1) * 8 +
-                  std::max<int64_t>(h.nc * h.nb, 1) * 8;
+        s = setup_block_rows(*m, ref, coords, cell_vertices, src, st);
     }
     if (s != SOPTX_OK) {
         std::string msg = g_last_error;
