@@ -363,6 +363,21 @@ soptx_status soptx_host_pair_tables(int dim, soptx_cell cell, int order, int64_t
                                     uint32_t *pair_meta, int32_t *record_cell, uint16_t *record_pair);
 
 /*
+ * Host-only sizes (no device work, usable without a GPU) of the tables by which
+ * k_block_rows assembles a 3D mesh off the box lattice, built exactly as
+ * soptx_mesh_create builds them: chunks, rows of 32 (pair, cell) records (with
+ * cached FP64 element matrices each row holds 2304 bytes of blocks beside them)
+ * and bytes of the chunk records.  *n_chunks = -1 where mesh creation builds
+ * none (2D, box lattices, general cells with FP32 element matrices, a node past
+ * the tables' or the shared memory's limits, tables of more than twice as many
+ * lanes as records).  Any output pointer may be NULL.
+ */
+soptx_status soptx_host_block_tables(int dim, soptx_cell cell, int order, int64_t n_vertices,
+                                     const double *coords, int64_t n_cells, const int32_t *cell_vertices,
+                                     soptx_elem_prec prec, int64_t *n_chunks, int64_t *n_rows,
+                                     int64_t *table_bytes);
+
+/*
  * Host-only inspection (no device work, usable without a GPU) of a node-owner
  * schedule of K(rho) = sum_e E(rho_e) K_e^0 (Sec. 2.2) on 3D meshes: a group of
  * nb lanes owns the d rows of one node and walks the node's cells as a chain.

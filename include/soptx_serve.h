@@ -105,8 +105,10 @@ soptx_status soptx_serve_submit(soptx_server srv, const soptx_request *req, uint
  * much room under hbm_cap_bytes (evicting idle meshes) before it builds a
  * job's mesh, then accounts the mesh's actual bytes: a job whose bound exceeds
  * the cap is still built once nothing else is resident, and fails with ENOMEM
- * only if its actual bytes do.  One pass over the cell array (the most cells
- * at a vertex bounds the padding of the pair kernel's tables).  Errors: EINVAL
+ * only if its actual bytes do.  It is 1.3 to 1.9 times the bytes of a large
+ * mesh (of a box lattice of order 1 up to 3 times).  Up to two passes over the
+ * cell array (whether all cells are equal; in 2D the most cells at a vertex,
+ * which bounds the padding of the pair kernel's tables).  Errors: EINVAL
  * for a NULL argument or a malformed mesh description, ENOMEM. */
 soptx_status soptx_serve_mesh_bytes_bound(const soptx_request *req, int64_t *bytes);
 

@@ -290,6 +290,19 @@ def host_pair_tables(cell, order, coords, cells, local_pair_bytes=False):
     return out
 
 
+def host_block_tables(cell, order, coords, cells, elem_prec="fp64"):
+    """Host-only sizes of the block-row kernel's tables (no GPU needed): None where mesh
+    creation builds none, else dict(n_chunks, n_rows (of 32 records), table_bytes)."""
+    coords = np.ascontiguousarray(coords, np.float64)
+    cells = np.ascontiguousarray(cells, np.int32)
+    nc, nr, nb = ctypes.c_int64(), ctypes.c_int64(), ctypes.c_int64()
+    N.check(N.lib().soptx_host_block_tables(
+        coords.shape[1], N.CELL[cell], int(order), coords.shape[0], coords.ctypes.data_as(ctypes.c_void_p),
+        cells.shape[0], cells.ctypes.data_as(ctypes.c_void_p) if cells.size else None, N.PREC[elem_prec],
+        ctypes.byref(nc), ctypes.byref(nr), ctypes.byref(nb)))
+    return None if nc.value < 0 else dict(n_chunks=nc.value, n_rows=nr.value, table_bytes=nb.value)
+
+
 def host_row_tables(cell, order, coords, cells):
     """Host-only node-owner schedule of 3D meshes with FP32 element matrices (no
     GPU needed): None where mesh creation builds none, else dict(nb, node_records

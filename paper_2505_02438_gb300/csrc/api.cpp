@@ -543,8 +543,35 @@ static bool build_row_tables(const HostMesh &h, RowTables &T)
     return true;
 }
 
+static BlockLimits block_limits(int nb, int src, int prec)
+{
+    BlockLimits L;
+    // FP32 blocks are symmetric only to their rounding: each is formed for its own place
+    L.sym = prec == SOPTX_ELEM_FP64;
+    // lanes that read the same block of K^0 beside one another (Q3 box 26x9x9: 202 -> 197 us)
+    L.by_code = src == kBlockUniform;
+    if (nb == 4) {
+        // linear tetrahedra meet 24 cells a node and 14 blocks: at the limits of the others
+        // a chunk has 7 nodes and the data-moving warp is the bottleneck (assembly of 1.1 M
+        // cells FP32 383 us, FP64 409; node-owner kernel before it 242 in FP32).  FP64: larger
+        // chunks, 289 (320 blocks and 300 cells 281, but slower than these below 100,000
+        // cells).  FP32: four CTAs of four warps, each with a data-moving warp, 250 us
+        // (100 blocks 273, three CTAs 260, two with 256 blocks 289)
+        L.blocks = src == kBlockContract ? 128 : 256;
+        L.cells = src == kBlockContract ? 140 : 256;
+    }
+    return L;
+}
+
+// Where a 3D mesh's blocks come from.
+static int block_source(soptx_path path, int prec)
+{
+    return path == SOPTX_PATH_UNIFORM ? kBlockUniform : prec == SOPTX_ELEM_FP32 ? kBlockContract : kBlockStream;
+}
+
 // Tables of the block-row kernel of 3D meshes (blockrows.cu).  The mesh keeps the
-// cached gather when its largest node does not fit in the tables or in shared memory.
+// cached gather when its largest node does not fit in the tables or in shared memory, or
+// when the tables would be mostly padding.
 static soptx_status build_block_rows(soptx_mesh_s &m, const RefElement &ref, const double *coords, const int32_t *cv,
                                      int src, cudaStream_t st)
 {
@@ -559,25 +586,11 @@ static soptx_status build_block_rows(soptx_mesh_s &m, const RefElement &ref, con
                 for (int kl = 0; kl < 9; kl++)
                     mf[((size_t)a * nb + b) * 12 + kl] = (float)ref.M[((size_t)kl * nb + a) * nb + b];
     }
-    BlockLimits L;
-    // FP32 blocks are symmetric only to their rounding: each is formed for its own place
-    L.sym = m.prec == SOPTX_ELEM_FP64;
-    // lanes that read the same block of K^0 beside one another (Q3 box 26x9x9: 202 -> 197 us)
-    L.by_code = src == kBlockUniform;
-    if (nb == 4) {
-        // linear tetrahedra meet 24 cells a node and 14 blocks: at the limits of the others
-        // a chunk has 7 nodes and the data-moving warp is the bottleneck (assembly of 1.1 M
-        // cells FP32 383 us, FP64 409; node-owner kernel before it 242 in FP32).  FP64: larger
-        // chunks, 289 (320 blocks and 300 cells 281, but slower than these below 100,000
-        // cells).  FP32: four CTAs of four warps, each with a data-moving warp, 250 us
-        // (100 blocks 273, three CTAs 260, two with 256 blocks 289)
-        L.blocks = src == kBlockContract ? 128 : 256;
-        L.cells = src == kBlockContract ? 140 : 256;
-    }
     BlockTables T;
-    if (!build_block_tables(h, coords, cv, L, T)) return SOPTX_OK;
+    if (!build_block_tables(h, coords, cv, block_limits(nb, src, m.prec), T) || !block_tables_small(T, h.nc, nb))
+        return SOPTX_OK;
     const int64_t smem = block_smem(src, nb, T);
-    if (smem > 220 * 1024) return SOPTX_OK;
+    if (smem > kBlockSmem) return SOPTX_OK;
     soptx_status s = SOPTX_OK;
     if (src == kBlockContract) {
         cell.assign((size_t)h.nc * 3, make_float4(0.f, 0.f, 0.f, 0.f));
@@ -896,10 +909,7 @@ soptx_status soptx_mesh_create(int dim, soptx_cell cell, int order, int64_t n_ve
         (!h.nonaffine || prec == SOPTX_ELEM_FP64)) {
         // 3D: the block rows of one matrix for all cells, of FP32 matrices of affine
         // cells contracted per call, or of the cached matrices
-        const int src = m->path == SOPTX_PATH_UNIFORM                   ? kBlockUniform
-                        : prec == SOPTX_ELEM_FP32          ? kBlockContract
-                                                                  : kBlockStream;
-        s = setup_block_rows(*m, ref, coords, cell_vertices, src, st);
+        s = setup_block_rows(*m, ref, coords, cell_vertices, block_source(m->path, prec), st);
     }
     if (s != SOPTX_OK) {
         std::string msg = g_last_error;
@@ -991,6 +1001,32 @@ soptx_status soptx_host_pair_tables(int dim, soptx_cell cell, int order, int64_t
         if (pair_meta && nt) std::memcpy(pair_meta, T.meta.data(), (size_t)nt * 32 * sizeof(uint32_t));
         if (record_cell && nrec) std::memcpy(record_cell, T.re.data(), (size_t)nrec * sizeof(int32_t));
         if (record_pair && nrec) std::memcpy(record_pair, T.rm.data(), (size_t)nrec * sizeof(uint16_t));
+    } catch (const std::bad_alloc &) {
+        SOPTX_FAIL(SOPTX_ENOMEM, "host allocation failed");
+    }
+    return SOPTX_OK;
+}
+
+soptx_status soptx_host_block_tables(int dim, soptx_cell cell, int order, int64_t n_vertices, const double *coords,
+                                     int64_t n_cells, const int32_t *cell_vertices, soptx_elem_prec prec,
+                                     int64_t *n_chunks, int64_t *n_rows, int64_t *table_bytes)
+{
+    RefElement ref;
+    HostMesh h;
+    if (n_chunks) *n_chunks = -1;
+    if (n_rows) *n_rows = 0;
+    if (table_bytes) *table_bytes = 0;
+    try {
+        const soptx_status s = plan_on_host(dim, cell, order, n_vertices, coords, n_cells, cell_vertices, ref, h);
+        if (s != SOPTX_OK || dim != 3 || h.lattice || h.nc == 0 || (h.nonaffine && prec != SOPTX_ELEM_FP64)) return s;
+        const int src = block_source(h.uniform ? SOPTX_PATH_UNIFORM : SOPTX_PATH_CACHED, prec);
+        BlockTables T;
+        if (!build_block_tables(h, coords, cell_vertices, block_limits(h.nb, src, prec), T) ||
+            !block_tables_small(T, h.nc, h.nb) || block_smem(src, h.nb, T) > kBlockSmem)
+            return SOPTX_OK;
+        if (n_chunks) *n_chunks = T.nchunks;
+        if (n_rows) *n_rows = T.rows;
+        if (table_bytes) *table_bytes = block_table_bytes(T);
     } catch (const std::bad_alloc &) {
         SOPTX_FAIL(SOPTX_ENOMEM, "host allocation failed");
     }

@@ -87,6 +87,8 @@ struct HostMesh {
 
 bool setup_host_mesh(int dim, int cell, int order, int64_t nv, const double *coords, int64_t nc,
                      const int32_t *cv, const RefElement &ref, HostMesh &hm, std::string &err);
+// Whether the mesh is uniform (HostMesh::uniform), from its description alone; false for ids out of range.
+bool uniform_cells(int dim, int cell, int64_t nv, const double *coords, int64_t nc, const int32_t *cv);
 void build_csr(const HostMesh &hm, std::vector<int64_t> &indptr, std::vector<int32_t> &indices);
 
 // ---------------------------------------------------------------- block rows
@@ -111,6 +113,18 @@ struct BlockTables {
 };
 bool build_block_tables(const HostMesh &hm, const double *coords, const int32_t *cv, const BlockLimits &lim,
                         BlockTables &T);
+// What the tables of a mesh may take (the admission bound of the server counts on it): twice
+// as many lanes as (pair, cell) records, 16 bytes a record, and a constant for small meshes.
+// Grids of any cell have 0.9 .. 1.2 lanes and 5 .. 10 bytes a record, Delaunay meshes of
+// random points 1.4 lanes; a mesh past it is assembled by the gather.
+inline int64_t block_lane_limit(int64_t nc, int nb) { return 2 * nc * nb * nb + (1 << 15); }
+inline int64_t block_byte_limit(int64_t nc, int nb) { return 16 * nc * nb * nb + (1 << 17); }
+inline int64_t block_table_bytes(const BlockTables &T) { return 4 * (int64_t)(T.blob.size() + T.coff.size()); }
+inline bool block_tables_small(const BlockTables &T, int64_t nc, int nb)
+{
+    return 32 * T.rows <= block_lane_limit(nc, nb) && block_table_bytes(T) <= block_byte_limit(nc, nb);
+}
+constexpr int64_t kBlockSmem = 220 * 1024;   // most shared memory of a CTA
 
 // ---------------------------------------------------------------- device mesh
 struct DeviceMesh {

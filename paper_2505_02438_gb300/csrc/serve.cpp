@@ -71,45 +71,50 @@ int64_t max_cells_at_vertex(const soptx_request &r, int nv)
 }
 
 // Upper bound of a mesh's device bytes from its input alone (every array of
-// soptx_mesh_create at its largest), used before the mesh exists.  The node-pair
-// tables of the pair kernel hold R records (a pair and one cell of it: at most
-// nb (nb + 1) / 2 per cell in 2D, nb^2 in 3D) padded per tile of 32 pairs to its
+// soptx_mesh_create at its largest), used before the mesh exists.  2D meshes hold the
+// node-pair tables of the pair kernel: R records (a pair and one cell of it: at most
+// nb (nb + 1) / 2 per cell) padded per tile of 32 pairs to its
 // largest count; within a window of pairs sorted by count a tile's largest is at
 // most the previous tile's smallest, so a window pads at most 32 times its
 // largest count (at most the most cells at a vertex, c) above its own records,
-// and windows hold 4096 pairs or more but the last.  In 2D with FP64 element
+// and windows hold 4096 pairs or more but the last.  With FP64 element
 // matrices each record also carries its 2 x 2 block (32 bytes).  3D meshes hold the
-// block-row kernel's chunk records instead: a chunk ends when its next node would
-// take it past 432 blocks, 110 cells or 192 nodes, so two neighbouring chunks pass one
-// of these together; each (pair, cell) has one lane of a record row (2 bytes, and with
-// FP64 element matrices its streamed block of 72), a pair's shares at most double it, and a
-// chunk's tiles pad 192 lanes by its most rows; 8 bytes per lane of a tile.
+// block-row kernel's chunk records, with cached FP64 matrices a block of 72 bytes for
+// each of their lanes; mesh creation takes them only within block_lane_limit and
+// block_byte_limit.  A mesh of equal cells holds one element matrix and no blocks.
 int64_t mesh_bytes_bound(const soptx_request &r)
 {
     static const int nb_tab[4][4] = {{0, 3, 6, 10}, {0, 4, 10, 20}, {0, 4, 9, 16}, {0, 8, 27, 64}};
-    static const int nv_tab[4] = {3, 4, 4, 8};
+    const int64_t nv = soptx::cell_nverts(r.cell), d = r.dim, ng = d * d + 1;
     const int64_t nb = nb_tab[r.cell][std::min(std::max(r.order, 1), 3)];
-    const int64_t ldof = r.dim * nb, nc = r.n_cells;
-    const int64_t ee = nc * ldof * ldof;          // >= nnz
-    const int64_t nn = r.n_vertices + nc * nb;    // >= nodes
-    const int64_t base = ee * 8 /* K_e (cached) */ + ee * 4 /* indices */ + nc * nb * nb * 2 /* pos */ +
-                         nc * nb * (4 + 4 + 4 + 1 + 8) /* cell_node, inc, inc_e, inc_a, partials */ +
-                         nn * r.dim * (8 + 8) + nn * 20 + nc * 120 + (1 << 20);
-    // general quadrilaterals and hexahedra: the geometry of every Gauss point
-    const int64_t points = nv_tab[r.cell] == (1 << r.dim) && r.cell != SOPTX_TET ? nb * (r.dim * r.dim + 1) * 8 : 0;
-    const int64_t c = std::min<int64_t>(max_cells_at_vertex(r, nv_tab[r.cell]), 1023);
+    const int64_t ldof = d * nb, nc = r.n_cells;
+    const bool tensor = !soptx::is_simplex(r.cell);
+    const bool uniform = r.coords && r.cell_vertices &&
+                         soptx::uniform_cells(r.dim, r.cell, r.n_vertices, r.coords, nc, r.cell_vertices);
+    const int64_t own = uniform ? 1 : nc;           // cells with matrices and geometry of their own
+    const int64_t nn = r.n_vertices + nc * (nb - nv);    // >= nodes
+    const int64_t pairs = nn + nc * nb * (nb - 1);      // >= row blocks
+    // K_e (FP64: float pairs), G and |det J| in FP64 and as float pairs (or in FP32)
+    int64_t bytes = own * (ldof * ldof * (r.prec == SOPTX_ELEM_FP64 ? 8 : 4) + 2 * ng * 8);
+    // general cells: corner coordinates, the geometry of every Gauss point
+    if (tensor) bytes += (uniform ? 0 : nc) * (nv * d * 8 + (r.prec == SOPTX_ELEM_FP64 ? nb * ng * 8 : 0));
+    bytes += 4 * d * d * pairs /* indices */ + nc * nb * nb * 2 /* pos */ +
+             nc * nb * (4 + 4 + 4 + 1 + 8) /* cell_node, inc, inc_e, inc_a, partials */ +
+             nn * d * (8 + 8) /* indptr, u */ + nn * (8 + 4) + nc * (8 + 8) /* moduli, block sums */;
+    // the tables of the reference element, rounding of small arrays
+    bytes += nb * nb * (d * d * 8 + 48 + 80) + 4 * nb * (nb * d + nv * d + 1) * 8 * 3 + (1 << 20);
     if (r.dim == 3) {
-        const int64_t rec = nc * nb * nb, chunks = 2 * (rec / 432 + nc * nb / 110 + nn / 192) + 1;
-        const int64_t lanes = 2 * rec + chunks * 192 * std::max<int64_t>(6, c / 32 + 1);
-        const int64_t per_lane = 2 + 8 + (r.prec == SOPTX_ELEM_FP64 ? 72 : 0);
-        return base + lanes * per_lane + nn * 8 + nc * nb * (4 + 48) + chunks * 64 + nc * points;
+        bytes += soptx::block_byte_limit(nc, (int)nb);
+        if (!uniform) bytes += r.prec == SOPTX_ELEM_FP64 ? 72 * soptx::block_lane_limit(nc, (int)nb) : 48 * nc;
+        return bytes;
     }
+    const int64_t c = std::min<int64_t>(max_cells_at_vertex(r, (int)nv), 1023);
     const int64_t rec = nc * (nb * (nb + 1) / 2);
     const int64_t windows = rec / 4096 + 1;
     const int64_t padded = rec + windows * 32 * c;
     const int64_t lanes = rec + windows * 32 + 7 * 32;   // and the last chunk of 8 tiles filled
     const int64_t per_rec = 4 + 2 + (r.prec == SOPTX_ELEM_FP64 ? 32 : 0);
-    return base + nc * points + padded * per_rec + lanes * 12 + (lanes / 32 + 32) * 4 + 64;
+    return bytes + nc * 32 + padded * per_rec + lanes * 12 + (lanes / 32 + 32) * 4 + 64;
 }
 
 }  // namespace

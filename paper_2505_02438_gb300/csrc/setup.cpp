@@ -80,6 +80,42 @@ std::array<int32_t, 4> sorted_key(const int32_t *v, int n)
     return k;
 }
 
+// The Jacobian of a cell at its first vertex and its largest entry; whether every corner of
+// it lies at x0 + sum_m bit_m J[:, m] (a simplex: always).
+bool cell_jacobian(int d, int cell, const double *coords, const int32_t *c, double (&J)[9], double &scale)
+{
+    const double *x0 = coords + (int64_t)c[0] * d;
+    scale = 0.0;
+    for (int m = 0; m < d; m++) {
+        const double *xm = coords + (int64_t)c[is_simplex(cell) ? m + 1 : (1 << m)] * d;
+        for (int i = 0; i < d; i++) {
+            J[i * d + m] = xm[i] - x0[i];
+            scale = std::max(scale, std::fabs(J[i * d + m]));
+        }
+    }
+    if (is_simplex(cell)) return true;
+    for (int v = 0; v < 1 << d; v++) {
+        const double *xv = coords + (int64_t)c[v] * d;
+        for (int i = 0; i < d; i++) {
+            double want = x0[i];
+            for (int m = 0; m < d; m++)
+                if ((v >> m) & 1) want += J[i * d + m];
+            if (std::fabs(xv[i] - want) > 1e-10 * scale) return false;
+        }
+    }
+    return true;
+}
+
+// Equal to within rounding of the coordinates (1e-14 of the largest entry).
+bool same_jacobian(int d, const double *J, const double *J0)
+{
+    double j0max = 0.0;
+    for (int q = 0; q < d * d; q++) j0max = std::max(j0max, std::fabs(J0[q]));
+    for (int q = 0; q < d * d; q++)
+        if (std::fabs(J[q] - J0[q]) > 1e-14 * j0max) return false;
+    return true;
+}
+
 bool geometry(HostMesh &hm, const double *coords, const int32_t *cv, std::string &err)
 {
     const int d = hm.dim, nvc = hm.nvc;
@@ -89,28 +125,10 @@ bool geometry(HostMesh &hm, const double *coords, const int32_t *cv, std::string
     double J0[9] = {0};
     for (int64_t e = 0; e < hm.nc; e++) {
         const int32_t *c = cv + e * nvc;
-        const double *x0 = coords + (int64_t)c[0] * d;
-        double J[9] = {0};   // J[i*d + m] = d x_i / d xi_m
-        for (int m = 0; m < d; m++) {
-            int vm = is_simplex(hm.cell) ? m + 1 : (1 << m);
-            const double *xm = coords + (int64_t)c[vm] * d;
-            for (int i = 0; i < d; i++) J[i * d + m] = xm[i] - x0[i];
-        }
-        double scale = 0.0;
-        for (int q = 0; q < d * d; q++) scale = std::max(scale, std::fabs(J[q]));
-        if (!is_simplex(hm.cell)) {
-            // affine check: every corner at x0 + sum_m bit_m J[:, m]; a general
-            // (bilinear / trilinear) cell is integrated by Gauss quadrature
-            bool affine = true;
-            for (int v = 0; v < nvc && affine; v++) {
-                const double *xv = coords + (int64_t)c[v] * d;
-                for (int i = 0; i < d; i++) {
-                    double want = x0[i];
-                    for (int m = 0; m < d; m++)
-                        if ((v >> m) & 1) want += J[i * d + m];
-                    if (std::fabs(xv[i] - want) > 1e-10 * scale) affine = false;
-                }
-            }
+        double J[9], scale;   // J[i*d + m] = d x_i / d xi_m
+        {
+            // a general (bilinear / trilinear) cell is integrated by Gauss quadrature
+            const bool affine = cell_jacobian(d, hm.cell, coords, c, J, scale);
             if (!affine) {
                 // the Jacobian at every corner (edges toward the corner's
                 // neighbours along each axis) must keep one sign
@@ -170,10 +188,7 @@ bool geometry(HostMesh &hm, const double *coords, const int32_t *cv, std::string
         if (e == 0) {
             std::memcpy(J0, J, sizeof(J));
         } else if (hm.uniform) {
-            double j0max = 0.0;
-            for (int q = 0; q < d * d; q++) j0max = std::max(j0max, std::fabs(J0[q]));
-            for (int q = 0; q < d * d; q++)
-                if (std::fabs(J[q] - J0[q]) > 1e-14 * j0max) hm.uniform = false;
+            hm.uniform = same_jacobian(d, J, J0);
         }
     }
     if (hm.nonaffine) {
@@ -248,6 +263,19 @@ void detect_lattice(HostMesh &hm, const double *coords, const int32_t *cv)
 }
 
 }  // namespace
+
+bool uniform_cells(int dim, int cell, int64_t nv, const double *coords, int64_t nc, const int32_t *cv)
+{
+    const int nvc = cell_nverts(cell);
+    double J[9], J0[9], scale;
+    for (int64_t e = 0; e < nc; e++) {
+        const int32_t *c = cv + e * nvc;
+        for (int v = 0; v < nvc; v++)
+            if (c[v] < 0 || c[v] >= nv) return false;
+        if (!cell_jacobian(dim, cell, coords, c, e ? J : J0, scale) || (e && !same_jacobian(dim, J, J0))) return false;
+    }
+    return nc > 0;
+}
 
 bool setup_host_mesh(int dim, int cell, int order, int64_t nv, const double *coords, int64_t nc,
                      const int32_t *cv, const RefElement &ref, HostMesh &hm, std::string &err)
