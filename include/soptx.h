@@ -156,7 +156,8 @@ soptx_status soptx_mesh_path(soptx_mesh mesh, soptx_path *path);
  *                  over the one matrix of a uniform mesh (k_contract_pairs in
  *                  2D, k_block_rows in 3D), 4 node pairs over the cached
  *                  element matrices of 3D cells, laid down in the kernel's
- *                  order (k_block_rows)
+ *                  order (k_block_rows; up to 4096 hexahedra of order 1 and
+ *                  256 P2 tetrahedra by the row gather all the same)
  *   *sensitivity : 0 box lattice (Walsh sectors), 1 fused into the row
  *                  gather, 2 strain energy at quadrature points
  *                  (k_strain_energy: affine cells; k_strain_corners and

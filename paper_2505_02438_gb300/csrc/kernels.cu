@@ -262,11 +262,21 @@ static int64_t kstride_of(const soptx_mesh_s &m)
     return m.path == SOPTX_PATH_CACHED ? (int64_t)m.h.ldof * m.h.ldof : 0;
 }
 
+// Meshes too small for the block rows over streamed matrices, whose chain from the ticket to
+// the stored rows takes 12 us however few the cells: the gather, us, against them: Q1
+// hexahedra 16 .. 810 cells 10.5 and 14.6, 6480 cells 21 and 22; P2 tetrahedra 12 cells 10.3
+// and 16.4, 96 cells 14.6 and 16.0, 900 cells 16.7 and 16.4.  (The other cells' gathers take
+// 19 .. 27 us on their smallest meshes.)
+static bool gather_is_shorter(const soptx_mesh_s &m)
+{
+    return m.d.bsrc == kBlockStream && m.h.nc <= (m.h.nb == 8 ? 4096 : m.h.nb == 10 ? 256 : 0);
+}
+
 cudaError_t launch_assemble(const soptx_mesh_s &m, const double *rho, double *vals, cudaStream_t st)
 {
     if (m.h.nn == 0 || m.h.nnz == 0) return cudaSuccess;
     if (m.path == SOPTX_PATH_LATTICE) return launch_lattice_assemble(m, rho, vals, st);
-    if (m.d.bchunks >= 0) return launch_block_rows(m, rho, vals, st);
+    if (m.d.bchunks >= 0 && !gather_is_shorter(m)) return launch_block_rows(m, rho, vals, st);
     if (m.d.contract || m.d.pcached || m.d.puniform) return launch_contract_assemble(m, rho, vals, st);
     return launch_gather(m, rho, nullptr, vals, nullptr, nullptr, nullptr, st);
 }
