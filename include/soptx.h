@@ -165,6 +165,22 @@ soptx_status soptx_mesh_path(soptx_mesh mesh, soptx_path *path);
  * Either pointer may be NULL.
  */
 soptx_status soptx_mesh_routes(soptx_mesh mesh, int32_t *assembly, int32_t *sensitivity);
+
+/*
+ * What served the mesh's latest calls, where a call has several ways:
+ *   *assembly : as above, of the latest assembly (-1: none yet); small meshes
+ *               may take the gather
+ *   *step     : one-call steps: 1 one launch of two clusters (small box
+ *               lattices), 2 launches of the assembly and the sensitivities,
+ *               3 the fused row gather
+ *   *backward : u-gradient from 1 the cells' forces, 2 the product over K(rho)
+ *               in the scratch, 3 the element matrices (no scratch)
+ *   *solve    : 1 one cooperative launch with K in shared memory, 2 the loop of
+ *               launches
+ * 0 before the first such call.  Any pointer may be NULL.
+ */
+soptx_status soptx_mesh_last_routes(soptx_mesh mesh, int32_t *assembly, int32_t *step, int32_t *backward,
+                                    int32_t *solve);
 soptx_status soptx_mesh_device_bytes(soptx_mesh mesh, int64_t *bytes);
 
 /*

@@ -81,6 +81,7 @@ SIGNATURES = {
     "soptx_mesh_copy_cell_nodes": (i32, [P, P, P]),
     "soptx_mesh_path": (i32, [P, Pi32]),
     "soptx_mesh_device_bytes": (i32, [P, Pi64]),
+    "soptx_mesh_last_routes": (i32, [P, Pi32, Pi32, Pi32, Pi32]),
     "soptx_mesh_routes": (i32, [P, Pi32, Pi32]),
     "soptx_assemble_K": (i32, [P, P, P, P]),
     "soptx_sensitivity": (i32, [P, P, P, P, P, P]),

@@ -88,6 +88,15 @@ class Mesh:
         return cls(wl.cell, wl.order, wl.coords, wl.cells, wl.E0, wl.Emin, wl.nu, wl.p, wl.plane_strain,
                    elem_prec or wl.elem_prec, stream)
 
+    def last_routes(self):
+        """What served the latest calls (soptx_mesh_last_routes), None before the first."""
+        r = [ctypes.c_int32() for _ in range(4)]
+        N.check(N.lib().soptx_mesh_last_routes(self._h, *(ctypes.byref(x) for x in r)))
+        names = ((None, "lattice", "gather", "contract", "pairs", "stream"), (None, "one launch", "launches", "fused"),
+                 (None, "forces", "product", "element matrices"), (None, "resident", "loop"))
+        return {k: n[x.value + (k == "assembly")]
+                for k, n, x in zip(("assembly", "step", "backward", "solve"), names, r)}
+
     def close(self):
         if getattr(self, "_h", None) is not None and self._h.value:
             N.lib().soptx_mesh_destroy(self._h)

@@ -1122,16 +1122,18 @@ soptx_status soptx_mesh_path(soptx_mesh m, soptx_path *path)
 soptx_status soptx_mesh_routes(soptx_mesh m, int32_t *assembly, int32_t *sensitivity)
 {
     if (!m) SOPTX_FAIL(SOPTX_EINVAL, "mesh is NULL");
-    if (assembly)
-        {
-        const auto &d = m->d;
-        *assembly = m->path == SOPTX_PATH_LATTICE                                                   ? 0
-                    : d.contract || (d.bchunks >= 0 && d.bsrc == kBlockContract)                ? 2
-                    : d.pcached || d.puniform || (d.bchunks >= 0 && d.bsrc == kBlockUniform) ? 3
-                    : d.bchunks >= 0                                                            ? 4
-                                                                                                : 1;
-    }
+    if (assembly) *assembly = assembly_route(*m);
     if (sensitivity) *sensitivity = (m->path == SOPTX_PATH_LATTICE && m->d.sectors) ? 0 : (m->d.strain ? 2 : 1);
+    return SOPTX_OK;
+}
+
+soptx_status soptx_mesh_last_routes(soptx_mesh m, int32_t *assembly, int32_t *step, int32_t *backward, int32_t *solve)
+{
+    if (!m) SOPTX_FAIL(SOPTX_EINVAL, "mesh is NULL");
+    if (assembly) *assembly = m->last_assembly;
+    if (step) *step = m->last_step;
+    if (backward) *backward = m->last_backward;
+    if (solve) *solve = m->last_solve;
     return SOPTX_OK;
 }
 
@@ -1305,7 +1307,9 @@ soptx_status soptx_compliance_vjp(soptx_mesh m, const double *d_rho, const doubl
         return cuda_status(cudaMemsetAsync(d_grad_u, 0, (size_t)m->h.ndof * sizeof(double), st),
                            "soptx_compliance_vjp");
     }
-    if (d_grad_u && d.kvals && vjp_matrix_free(*m))
+    const bool forces = d_grad_u && d.kvals && vjp_matrix_free(*m);
+    if (d_grad_u) m->last_backward = forces ? 1 : d.kvals ? 2 : 3;
+    if (forces)
         return cuda_status(launch_vjp(*m, d_rho, d_u, d_gout, d_grad_rho, d_grad_u, (float2 *)d.kvals, st),
                            "soptx_compliance_vjp");
     if (d_grad_u && d.kvals) {

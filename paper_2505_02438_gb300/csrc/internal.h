@@ -238,12 +238,15 @@ struct soptx_mesh_s {
     int prec = SOPTX_ELEM_FP64;
     soptx_path path = SOPTX_PATH_CACHED;
     int64_t device_bytes = 0;
+    // what served the latest calls (soptx_mesh_last_routes)
+    mutable int32_t last_assembly = -1, last_step = 0, last_backward = 0, last_solve = 0;
     mutable uint32_t lattice_gen = 0;   // calls of the 3D lattice assembly (marks the out-of-range flag)
 };
 
 namespace soptx {
 // ---------------------------------------------------------------- launchers (kernels.cu)
 cudaError_t launch_element_matrices(const soptx_mesh_s &m, int64_t n_elems, cudaStream_t st);
+int32_t assembly_route(const soptx_mesh_s &m);   // soptx_mesh_routes
 cudaError_t launch_assemble(const soptx_mesh_s &m, const double *rho, double *vals, cudaStream_t st);
 cudaError_t launch_sensitivity(const soptx_mesh_s &m, const double *rho, const double *u, double *dc,
                                double *c, double scale, const double *gscale, cudaStream_t st);

@@ -272,12 +272,23 @@ static bool gather_is_shorter(const soptx_mesh_s &m)
     return m.d.bsrc == kBlockStream && m.h.nc <= (m.h.nb == 8 ? 4096 : m.h.nb == 10 ? 256 : 0);
 }
 
+int32_t assembly_route(const soptx_mesh_s &m)
+{
+    const auto &d = m.d;
+    if (m.path == SOPTX_PATH_LATTICE) return 0;
+    if (d.contract || (d.bchunks >= 0 && d.bsrc == kBlockContract)) return 2;
+    if (d.pcached || d.puniform || (d.bchunks >= 0 && d.bsrc == kBlockUniform)) return 3;
+    return d.bchunks >= 0 ? 4 : 1;
+}
+
 cudaError_t launch_assemble(const soptx_mesh_s &m, const double *rho, double *vals, cudaStream_t st)
 {
     if (m.h.nn == 0 || m.h.nnz == 0) return cudaSuccess;
+    const bool rows = m.d.bchunks >= 0 && !gather_is_shorter(m), pairs = m.d.contract || m.d.pcached || m.d.puniform;
+    m.last_assembly = rows || pairs || m.path == SOPTX_PATH_LATTICE ? assembly_route(m) : 1;
     if (m.path == SOPTX_PATH_LATTICE) return launch_lattice_assemble(m, rho, vals, st);
-    if (m.d.bchunks >= 0 && !gather_is_shorter(m)) return launch_block_rows(m, rho, vals, st);
-    if (m.d.contract || m.d.pcached || m.d.puniform) return launch_contract_assemble(m, rho, vals, st);
+    if (rows) return launch_block_rows(m, rho, vals, st);
+    if (pairs) return launch_contract_assemble(m, rho, vals, st);
     return launch_gather(m, rho, nullptr, vals, nullptr, nullptr, nullptr, st);
 }
 
@@ -297,6 +308,7 @@ cudaError_t launch_sensitivity(const soptx_mesh_s &m, const double *rho, const d
 cudaError_t launch_step(const soptx_mesh_s &m, const double *rho, const double *u, double *vals, double *dc,
                         double *c, cudaStream_t st, const double *gscale)
 {
+    m.last_step = 2;
     if (m.path == SOPTX_PATH_LATTICE && m.d.sectors && m.h.nc > 0)
         return launch_lattice_step(m, rho, u, vals, dc, c, st, gscale);
     if (m.d.strain && m.d.side && m.h.nc > 0 && m.h.nnz > 0 &&
@@ -341,6 +353,8 @@ cudaError_t launch_step(const soptx_mesh_s &m, const double *rho, const double *
         if (err != cudaSuccess) return err;
         return launch_sensitivity(m, rho, u, dc, c, -1.0, gscale, st);
     }
+    m.last_step = 3;
+    m.last_assembly = 1;
     return launch_gather(m, rho, u, m.h.nnz > 0 ? vals : nullptr, dc, c, gscale, st);
 }
 

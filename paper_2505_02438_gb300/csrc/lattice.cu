@@ -1109,6 +1109,7 @@ cudaError_t launch_lattice_step(const soptx_mesh_s &m, const double *rho, const 
         const cudaError_t err = m.h.dim == 3            ? launch_single<3, 8>(m, rho, u, vals, dc, c, st, gscale)
                                 : m.h.nn > kSingleWide ? launch_single<2, 16>(m, rho, u, vals, dc, c, st, gscale)
                                                        : launch_single<2, 8>(m, rho, u, vals, dc, c, st, gscale);
+        if (err == cudaSuccess) m.last_step = 1;
         if (err != cudaErrorLaunchOutOfResources && err != cudaErrorInvalidClusterSize) return err;
         cudaGetLastError();   // no room for a cluster of 16: the launches below
     }

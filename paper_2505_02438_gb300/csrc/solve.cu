@@ -488,6 +488,7 @@ soptx_status soptx_solve_cg(soptx_mesh m, const double *d_vals, const uint8_t *d
         e = cg_resident_run(*m, d_vals, d_fixed, diag, d_u, r, z, pv, S + 4, o->check_every, o->max_iter, o->rtol * r0,
                             st, &out, &launched);
         if (launched) {
+            m->last_solve = 1;
             if (e != cudaSuccess) return cuda_fail(e, "soptx_solve_cg");
             if (out.error) SOPTX_FAIL(SOPTX_ECUDA, "soptx_solve_cg: a wait between the blocks ran out");
             res->iterations = out.it;
@@ -498,6 +499,7 @@ soptx_status soptx_solve_cg(soptx_mesh m, const double *d_vals, const uint8_t *d
         e = cudaSuccess;
         cudaGetLastError();   // refused: the loop below
     }
+    m->last_solve = 2;
     // One CG iteration: three dependent launches (each is scheduled while the one
     // before it finishes and waits for it before reading anything).
     auto iteration = [&](int it_, cudaStream_t s_) -> cudaError_t {
