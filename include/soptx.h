@@ -193,9 +193,11 @@ soptx_status soptx_mesh_device_bytes(soptx_mesh mesh, int64_t *bytes);
  * absolute element contributions of the exact value (FP64 element matrices).
  * The order depends on the path: on a general mesh each value is the sum of
  * its element contributions in ascending element order (float-pair
- * accumulation), on a 3D mesh in up to 32 such shares added in a fixed tree; on a box lattice it is the reference block entry times a
- * signed sum of the (at most 2^d) moduli of the cells the two nodes share,
- * formed by per-axis sums and differences.
+ * accumulation), on a 3D mesh in up to 32 such shares added in a fixed tree; on
+ * a box lattice it is the reference block entry times a signed sum of the (at
+ * most 2^d) moduli of the cells the two nodes share, formed by per-axis sums
+ * and differences.  Float pairs have an absolute step of 2^-149: values below
+ * about 1e-30 have fewer correct digits.
  */
 soptx_status soptx_assemble_K(soptx_mesh mesh, const double *d_rho, double *d_vals, void *stream);
 
@@ -212,11 +214,12 @@ soptx_status soptx_sensitivity(soptx_mesh mesh, const double *d_rho, const doubl
 
 /* One pass that produces both K(rho) and the sensitivities (the per-iteration
  * step); same arguments and results as the two calls above: K and dc bitwise,
- * c the same fixed-order sum of block partials (on 2D meshes of affine cells
- * other than box lattices, and 3D ones, over a few blocks per SM, so its last
- * bits may differ from the separate call's when the mesh has more cells than
- * those blocks hold).  On a 2D box lattice the sensitivities run on a second, mesh-owned
- * stream beside the assembly; on other meshes they run first on that stream
+ * c the same fixed-order sum of block partials (on meshes other than box
+ * lattices over a few blocks per SM, so its last bits may differ from the
+ * separate call's when the mesh has more cells than those blocks hold).  Small
+ * box lattices (1536 cells in 2D, 1024 in 3D) take one launch.  On a larger 2D
+ * box lattice the sensitivities run on a second, mesh-owned stream beside the
+ * assembly; on other meshes they run first on that stream
  * (created at the highest stream priority), a few blocks per SM, beside the
  * assembly on `stream` (the stream and two events are made by the first such
  * call); everything is ordered on `stream` when the call returns. */

@@ -58,9 +58,9 @@ static cudaError_t ensure_side(soptx_mesh_s &m)
     if (d.side) return cudaSuccess;
     cudaStream_t side = nullptr;
     cudaEvent_t ev[2] = {};
-    // meshes with the strain-energy sensitivities run their assembly (3D) or
-    // their sensitivities (2D) on this stream in the one-call step, at the
-    // highest priority (see launch_step)
+    // meshes with the strain-energy sensitivities run them (or, where the gather assembles
+    // affine cells, the assembly) on this stream in the one-call step, at the highest
+    // priority (see launch_step)
     int least = 0, greatest = 0;
     cudaError_t e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
     if (e == cudaSuccess)

@@ -78,7 +78,7 @@ struct BlockArgs {
     int64_t nchunks;
     unsigned *__restrict__ ticket;        // [0] chunks handed out, [1] CTAs done (both zero between calls)
     volatile unsigned *expired;           // host memory: set when a wait ran out (the next call reports it)
-    int tries;                            // limit of a wait
+    int tries;                            // limit of the data-moving warp's waits
     const uint4 *__restrict__ blob;
     const uint32_t *__restrict__ coff;    // [nchunks + 1] chunk starts in 16-byte units
     int max_blob, max_cells, max_stage, cell_bits;   // 16-byte units, cells, values; of a record
@@ -114,10 +114,11 @@ __device__ __forceinline__ void bulk_store(double *gdst, const double *ssrc, uin
                  : "memory");
 }
 
-// Shared-memory barriers (mbarrier).  Every wait is bounded: after BlockArgs::tries tries
-// (kBlockWaitTries) of up to 20 us each the whole warp gives up, raises the error word and
-// leaves; the others' waits run out after it, and the data-moving warp still waits, with
-// the full limit, for the copies that it has in flight.
+// Shared-memory barriers (mbarrier).  Every wait is bounded: after kBlockWaitTries tries (the
+// data-moving warp: BlockArgs::tries, the same but in tests) of up to 20 us each the whole
+// warp gives up, raises the error word and leaves.  The data-moving warp then ends the
+// chunks of the others and still waits, with the full limit, for the copies that it has in
+// flight; when another warp gives up, its waits run out after it.
 __device__ __forceinline__ void mbar_init(uint64_t *b, unsigned count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(b)), "r"(count) : "memory");
@@ -388,8 +389,9 @@ __global__ void __launch_bounds__(32 * (W + 1), MINB) k_block_rows(const BlockAr
             if (ok) gather_cells(record(0), cbuf);
             cp_async_wait_all();
         }
-        open(0, more && ok);
         int q = 0, last = more ? 1 : 0;   // (k + 1) mod 3; chunks known to exist
+        more = more && ok;
+        open(0, more);
         for (int k = 0; ok && k < last + 2; k++) {
             const int s = k & 1;
             q = q == 2 ? 0 : q + 1;
@@ -420,6 +422,11 @@ __global__ void __launch_bounds__(32 * (W + 1), MINB) k_block_rows(const BlockAr
         }
         if (!ok) {
             raise();
+            __syncwarp();
+            if (more && lane == 0) {   // the next chunk, which is not there
+                s_more[q] = 0;
+                mbar_arrive(&s_full[q]);
+            }
             while (landed < issued && wait_record(kBlockWaitTries)) {
             }
         }
@@ -442,7 +449,7 @@ __global__ void __launch_bounds__(32 * (W + 1), MINB) k_block_rows(const BlockAr
     unsigned pq = 0;   // parity of s_full[q]
     for (int k = 0;; k++) {
         const int s = k & 1;
-        if (!mbar_wait(&s_full[q], pq, A.tries)) return raise();
+        if (!mbar_wait(&s_full[q], pq, kBlockWaitTries)) return raise();
         if (!s_more[q]) return;
         const uint32_t *B = reinterpret_cast<const uint32_t *>(blobs + (k & 3) * A.max_blob);
         const unsigned char *const cb = cbuf + q * cstride;
@@ -536,7 +543,7 @@ __global__ void __launch_bounds__(32 * (W + 1), MINB) k_block_rows(const BlockAr
             for (int p = 0; p < 9; p++) big = max_nan(big, fabsf(v[p].x));
             bad |= !(big <= FLT_MAX);
             if (!free) {
-                if (!mbar_wait(&s_free[s], (k >> 1) & 1, A.tries)) return raise();
+                if (!mbar_wait(&s_free[s], (k >> 1) & 1, kBlockWaitTries)) return raise();
                 free = true;
             }
             const uint32_t o1 = pr.x & 0xffffu;

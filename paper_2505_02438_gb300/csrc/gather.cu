@@ -583,8 +583,8 @@ cudaError_t gather_t(const soptx_mesh_s &m, const double *rho, double *vals, boo
     // (80 registers); the assembly alone fits in 64 registers at 4 CTAs per SM.
     if constexpr (D == 3) {
         if (nb == 10) {   // P2 tetrahedra
-            if (sens) SOPTX_ROWS(10, true, 2, 6, 5, 3);   // 2 nodes x 3 rows x 5 lanes, 6 rounds
-            SOPTX_ROWS(10, false, 1, 3, 10, 4);           // 1 node x 3 rows x 10 lanes, 3 rounds
+            // (never with sensitivities: affine cells take k_strain_energy)
+            if (!sens) SOPTX_ROWS(10, false, 1, 3, 10, 4);   // 1 node x 3 rows x 10 lanes, 3 rounds
         }
         if (nb == 8) {    // Q1 hexahedra
             if (sens) SOPTX_ROWS(8, true, 2, 6, 4, 3);    // 2 nodes x 3 rows x 4 lanes, 6 rounds
@@ -592,8 +592,7 @@ cudaError_t gather_t(const soptx_mesh_s &m, const double *rho, double *vals, boo
         }
     } else {
         if (nb == 10) {   // P3 triangles: 4 nodes x 2 rows x 4 lanes, 5 rounds
-            if (sens) SOPTX_ROWS(10, true, 4, 5, 4, 3);
-            SOPTX_ROWS(10, false, 4, 5, 4, 4);
+            if (!sens) SOPTX_ROWS(10, false, 4, 5, 4, 4);
         }
         if (nb == 4) {    // Q1 quadrilaterals: 4 nodes x 2 rows x 4 lanes, 2 rounds
             if (sens) SOPTX_ROWS(4, true, 4, 2, 4, 3);
