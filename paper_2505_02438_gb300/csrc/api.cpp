@@ -619,9 +619,17 @@ static soptx_status build_block_rows(soptx_mesh_s &m, const RefElement &ref, con
     if (s == SOPTX_OK && !mf.empty()) s = upload(&m.d.bM, mf, st, m.device_bytes, "reference integrals (FP32)");
     if (s == SOPTX_OK && !blk.empty()) s = upload(&m.d.bkblk, blk, st, m.device_bytes, "element matrix blocks");
     if (s == SOPTX_OK) {
-        uint32_t *p = nullptr;   // (32-bit words, a whole number of 16-byte units)
-        s = upload(&p, T.blob, st, m.device_bytes, "chunk records");
-        m.d.bblob = reinterpret_cast<uint4 *>(p);
+        // (32-bit words, a whole number of 16-byte units)
+        cudaError_t e = dev_alloc((void **)&m.d.bblob, (size_t)T.words * 4);
+        int64_t at = 0;
+        for (const auto &part : T.blob) {
+            if (e == cudaSuccess && !part.empty())
+                e = cudaMemcpyAsync((uint32_t *)m.d.bblob + at, part.data(), part.size() * 4, cudaMemcpyHostToDevice, st);
+            at += (int64_t)part.size();
+        }
+        s = cuda_status(e, "chunk records");
+        if (s == SOPTX_OK) m.device_bytes += std::max<int64_t>(T.words * 4, 16);
+        else cudaGetLastError();
     }
     if (s == SOPTX_OK) s = upload(&m.d.bcoff, T.coff, st, m.device_bytes, "chunk offsets");
     if (s == SOPTX_OK) s = upload(&m.d.cticket, std::vector<unsigned>(2, 0u), st, m.device_bytes, "chunk counter");

@@ -6,7 +6,6 @@
 #include <cmath>
 #include <cstring>
 #include <new>
-#include <system_error>
 #include <thread>
 
 #include "internal.h"
@@ -43,34 +42,71 @@ uint64_t hilbert_index(uint32_t *x, int b, int d)
     return h;
 }
 
+int64_t shares_for(int64_t items, int64_t least)
+{
+    return std::max<int64_t>(1, std::min<int64_t>({16, (int64_t)std::thread::hardware_concurrency(), items / least}));
+}
+
+// f(0) .. f(n - 1), one per thread; those whose thread cannot be had run in this one.  f does not throw.
+template <typename F>
+void in_threads(int64_t n, const F &f)
+{
+    std::vector<std::thread> pool;
+    int64_t here = 1;
+    try {
+        pool.reserve((size_t)n);
+        for (; here < n; here++) pool.emplace_back(f, here);
+    } catch (const std::exception &) {
+    }
+    f(0);
+    for (int64_t k = here; k < n; k++) f(k);
+    for (auto &t : pool) t.join();
+}
+
 // Processing order of the nodes: by the place of their first cell along a
 // Hilbert curve through the cells' centroids, so consecutive nodes are close
 // together, share most of their cells and are each other's neighbours.
 std::vector<int32_t> node_order(const HostMesh &h, const double *coords, const int32_t *cv)
 {
     const int d = h.dim, nvc = h.nvc, bits = d == 2 ? 16 : 10;
-    std::vector<double> cen((size_t)h.nc * d);
+    const int64_t shares = shares_for(h.nc, 4096);
+    std::vector<double> cen((size_t)h.nc * d), lo_s((size_t)shares * d, HUGE_VAL), hi_s((size_t)shares * d, -HUGE_VAL);
+    in_threads(shares, [&](int64_t k) {
+        for (int64_t e = h.nc * k / shares; e < h.nc * (k + 1) / shares; e++)
+            for (int i = 0; i < d; i++) {
+                double s = 0.0;
+                for (int v = 0; v < nvc; v++) s += coords[(int64_t)cv[e * nvc + v] * d + i];
+                s /= nvc;
+                cen[(size_t)e * d + i] = s;
+                lo_s[(size_t)k * d + i] = std::min(lo_s[(size_t)k * d + i], s);
+                hi_s[(size_t)k * d + i] = std::max(hi_s[(size_t)k * d + i], s);
+            }
+    });
     double lo[3] = {0, 0, 0}, ext = 0.0;
     for (int i = 0; i < d; i++) {
         double a = HUGE_VAL, b = -HUGE_VAL;
-        for (int64_t e = 0; e < h.nc; e++) {
-            double s = 0.0;
-            for (int v = 0; v < nvc; v++) s += coords[(int64_t)cv[e * nvc + v] * d + i];
-            cen[(size_t)e * d + i] = s / nvc;
-            a = std::min(a, s / nvc);
-            b = std::max(b, s / nvc);
+        for (int64_t k = 0; k < shares; k++) {
+            a = std::min(a, lo_s[(size_t)k * d + i]);
+            b = std::max(b, hi_s[(size_t)k * d + i]);
         }
         lo[i] = a;
         ext = std::max(ext, b - a);
     }
     const double scale = ext > 0.0 ? ((1u << bits) - 1) / ext : 0.0;
     std::vector<std::pair<uint64_t, int32_t>> key((size_t)h.nc);
-    for (int64_t e = 0; e < h.nc; e++) {
-        uint32_t x[3] = {0, 0, 0};
-        for (int i = 0; i < d; i++) x[i] = (uint32_t)((cen[(size_t)e * d + i] - lo[i]) * scale);
-        key[(size_t)e] = {hilbert_index(x, bits, d), (int32_t)e};
-    }
-    std::sort(key.begin(), key.end());
+    in_threads(shares, [&](int64_t k) {
+        for (int64_t e = h.nc * k / shares; e < h.nc * (k + 1) / shares; e++) {
+            uint32_t x[3] = {0, 0, 0};
+            for (int i = 0; i < d; i++) x[i] = (uint32_t)((cen[(size_t)e * d + i] - lo[i]) * scale);
+            key[(size_t)e] = {hilbert_index(x, bits, d), (int32_t)e};
+        }
+        std::sort(key.begin() + h.nc * k / shares, key.begin() + h.nc * (k + 1) / shares);
+    });
+    for (int64_t w = 1; w < shares; w *= 2)   // merges of sorted shares
+        in_threads((shares + 2 * w - 1) / (2 * w), [&](int64_t k) {
+            auto at = [&](int64_t q) { return key.begin() + h.nc * std::min(q, shares) / shares; };
+            std::inplace_merge(at(2 * w * k), at(2 * w * k + w), at(2 * w * k + 2 * w));
+        });
     std::vector<int32_t> order;
     order.reserve((size_t)h.nn);
     std::vector<char> seen((size_t)h.nn, 0);
@@ -93,6 +129,7 @@ bool build_chunks(const HostMesh &h, const BlockLimits &L, const std::vector<int
 {
     const int d = h.dim, nb = h.nb;
     T.coff.push_back(0);
+    T.blob.resize(1);
     std::vector<int32_t> cell_chunk((size_t)h.nc, -1), cell_loc((size_t)h.nc, 0);
     std::vector<int32_t> cells;
     struct Pair {
@@ -201,7 +238,7 @@ bool build_chunks(const HostMesh &h, const BlockLimits &L, const std::vector<int
                 return kx != ky ? kx < ky : (prec[pairs[x].r0] >> 16) < (prec[pairs[y].r0] >> 16);
             });
         // lanes: (pair, share) in tiles of 32
-        std::vector<uint32_t> &B = T.blob;
+        std::vector<uint32_t> &B = T.blob[0];
         const size_t b0 = B.size();
         size_t lanes = 0;
         for (auto &w : pairs) lanes += (size_t)1 << w.lg;
@@ -336,8 +373,7 @@ bool build_block_tables(const HostMesh &h, const double *coords, const int32_t *
         T.nchunks = chunk + 1;
     }
     // their records, in shares of consecutive chunks, one per thread
-    const int64_t shares = std::max<int64_t>(
-        1, std::min<int64_t>({8, (int64_t)std::thread::hardware_concurrency(), T.nchunks / 64}));
+    const int64_t shares = shares_for(T.nchunks, 64);
     std::vector<BlockTables> part((size_t)shares);
     std::vector<char> good((size_t)shares, 0);   // 0: failed, 1: built, 2: out of memory
     auto run = [&](int64_t k) {
@@ -349,28 +385,20 @@ bool build_block_tables(const HostMesh &h, const double *coords, const int32_t *
             good[(size_t)k] = 2;
         }
     };
-    std::vector<std::thread> pool;
-    int64_t here = 0;   // shares from this one on run in this thread
-    try {
-        for (here = 1; here < shares; here++) pool.emplace_back(run, here);
-    } catch (const std::system_error &) {
-    }
-    run(0);
-    for (int64_t k = here; k < shares; k++) run(k);
-    for (auto &t : pool) t.join();
+    in_threads(shares, run);
     T.cell_bits = cell_bits;
     T.coff.push_back(0);
     for (int64_t k = 0; k < shares; k++) {
         BlockTables &P = part[(size_t)k];
         if (good[(size_t)k] == 2) throw std::bad_alloc();
         if (!good[(size_t)k] || T.rows + P.rows > (int64_t)UINT32_MAX ||
-            (T.blob.size() + P.blob.size()) / 4 > (size_t)UINT32_MAX)
+            (T.words + (int64_t)P.blob[0].size()) / 4 > (int64_t)UINT32_MAX)
             return false;
         const uint32_t base = T.coff.back();
-        for (size_t c = 0; c + 1 < P.coff.size(); c++) P.blob[4 * (size_t)P.coff[c] + 4] += (uint32_t)T.rows;
+        for (size_t c = 0; c + 1 < P.coff.size(); c++) P.blob[0][4 * (size_t)P.coff[c] + 4] += (uint32_t)T.rows;
         for (size_t c = 1; c < P.coff.size(); c++) T.coff.push_back(base + P.coff[c]);
-        T.blob.insert(T.blob.end(), P.blob.begin(), P.blob.end());
-        std::vector<uint32_t>().swap(P.blob);
+        T.words += (int64_t)P.blob[0].size();
+        T.blob.push_back(std::move(P.blob[0]));
         T.rows += P.rows;
         T.max_blob = std::max(T.max_blob, P.max_blob);
         T.max_cells = std::max(T.max_cells, P.max_cells);

@@ -104,7 +104,10 @@ struct BlockLimits {
     int cap = 6;         // cells per lane before a pair is shared by several lanes
 };
 struct BlockTables {
-    std::vector<uint32_t> blob;   // the chunks' records, each a whole number of 16-byte units
+    // the chunks' records, each a whole number of 16-byte units, in the parts that the threads
+    // built, one after another (joined on the device: a copy here took a fifth of the tables' time)
+    std::vector<std::vector<uint32_t>> blob;
+    int64_t words = 0;            // in all parts
     std::vector<uint32_t> coff;   // [nchunks + 1] their starts in 16-byte units
     int64_t nchunks = 0, rows = 0;
     int cell_bits = 0;            // bits of a record that name the chunk's cell
@@ -119,7 +122,7 @@ bool build_block_tables(const HostMesh &hm, const double *coords, const int32_t 
 // random points 1.4 lanes; a mesh past it is assembled by the gather.
 inline int64_t block_lane_limit(int64_t nc, int nb) { return 2 * nc * nb * nb + (1 << 15); }
 inline int64_t block_byte_limit(int64_t nc, int nb) { return 16 * nc * nb * nb + (1 << 17); }
-inline int64_t block_table_bytes(const BlockTables &T) { return 4 * (int64_t)(T.blob.size() + T.coff.size()); }
+inline int64_t block_table_bytes(const BlockTables &T) { return 4 * (T.words + (int64_t)T.coff.size()); }
 inline bool block_tables_small(const BlockTables &T, int64_t nc, int nb)
 {
     return 32 * T.rows <= block_lane_limit(nc, nb) && block_table_bytes(T) <= block_byte_limit(nc, nb);
