@@ -28,8 +28,10 @@
 // the cache, a node-owner contraction, the pair kernel without symmetry): P2 tets
 // 60x20x20 FP64 350 -> 296, FP32 283 -> 216; jittered hexahedra Q1 120x40x40 337 -> 249,
 // Q2 40x14x14 316 -> 166, Q3 26x9x9 699 -> 265; boxes Q2 195 -> 118, Q3 282 -> 197.
-// What bounds it: kContract the FP32 instructions at 16 warps per SM (65% issue), kUniform
-// the L1 data pipe (the blocks of K^0 and the staged rows), kStream DRAM (4.9 TB/s).
+// What bounds it (a capture each): kContract the FP32 instructions at 16 warps per SM (65%
+// issue); kUniform no pipe alone (issue 52%, L1 data pipe 53%, the conversions' FP64 pipe
+// 50%) but the latency of K^0's blocks and the dependences at those warps; kStream the latency
+// of its one read of the blocks, at 4.9 TB/s.
 //
 // A block K_e^0[(a,.),(b,.)] comes from one of the following (SRC):
 //   kContract : FP32 element matrices of affine cells, never stored: the

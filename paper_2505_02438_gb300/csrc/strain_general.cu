@@ -90,7 +90,9 @@ __device__ __forceinline__ void put_cell(const GeneralArgs &A, int64_t e, double
 // over the cached matrices 3.2e-15).  The derivative of component i along axis m at the
 // signs s of the other axes lies at us[((m D + i) 2^(D-1) + s) kThreads + thread]: in
 // registers, with the points unrolled, the kernel waited on instruction fetches (80 us in
-// place of 68 on 192,000 hexahedra).
+// place of 68 on 192,000 hexahedra).  Bound by instruction issue (55% of the slots, 45% with
+// the last wave) and the latency of the geometry's loads at 15 warps per SM, 36 KB of shared
+// memory a block; the 123 MB of geometry alone take 18 us.
 template <int D>
 __global__ void __launch_bounds__(kThreads, 5) k_strain_corners(const GeneralArgs A)
 {
@@ -209,9 +211,9 @@ __device__ __forceinline__ double density(const double (&gu)[3][3], double lam, 
 // the rule one of n = K + 1 points, so the reference gradient at the n^d points is d passes
 // of 1D contractions through shared memory.  A lane per point (two for the 64 of a
 // hexahedron), its rows of the 1D tables in registers; a warp holds 3 quadrilaterals of 9
-// points, 2 of 16 or one hexahedron.  Bound by the FP64 pipe (16 cycles of it an instruction).
-// (A thread per quadrilateral: 111 us in place of 68 on 97,000 cells of order 2, and 56 us
-// on any small mesh of order 3, a chain of 1300 operations.)
+// points, 2 of 16 or one hexahedron.  Bound by the FP64 pipe (81 .. 84% busy, 16 cycles of it
+// an instruction).  A thread per quadrilateral took 111 us on 97,000 cells of order 2 (103
+// here) and 56 us on any small mesh of order 3, a chain of 1300 operations (9 here).
 template <int D, int K>
 __global__ void __launch_bounds__(kThreads) k_strain_tensor(const GeneralArgs A)
 {
@@ -248,117 +250,117 @@ __global__ void __launch_bounds__(kThreads) k_strain_tensor(const GeneralArgs A)
     const int64_t take = (int64_t)NC * A.rounds;
     for (int64_t c0 = ((int64_t)blockIdx.x * (kThreads / 32) + warp) * take; c0 < A.nc;
          c0 += (int64_t)gridDim.x * (kThreads / 32) * take) {
-      double mys = 0.0;   // of cell c0 + lane
-      for (int j = 0; j < A.rounds && c0 + j * NC < A.nc; j++) {
-        const int64_t e = c0 + j * NC + gi;
-        const bool on = gi < NC && e < A.nc;
-        __syncwarp();
-        if (on)
-#pragma unroll
-            for (int p = 0; p < NP; p++) {
-                const int64_t nd = __ldg(A.cell_node + e * P + r + GL * p);
-#pragma unroll
-                for (int i = 0; i < D; i++) us[i * P + lat[p]] = __ldg(A.u + D * nd + i);
-            }
-        __syncwarp();
-        // first index: av, ad at (q1, b2, b3) = sum_b1 l, l'_(b1)(q1) u(b1, b2, b3)
-        if (on)
-#pragma unroll
-            for (int p = 0; p < NP; p++)
-#pragma unroll
-                for (int i = 0; i < D; i++) {
-                    const int o = i * P + r + GL * p;
-                    double sv = 0.0, sd = 0.0;
-#pragma unroll
-                    for (int b = 0; b < n; b++) {
-                        const double x = us[o - q1 + b];
-                        sv = fma(v1[b], x, sv);
-                        sd = fma(d1[b], x, sd);
-                    }
-                    av[o] = sv;
-                    ad[o] = sd;
-                }
-        __syncwarp();
-        double s = 0.0;
-        if constexpr (D == 2) {
-            if (on) {
-                double U[2][2], gu[2][2], G[NG];
-                const double *gp = reinterpret_cast<const double *>(A.geo) + e * P * NG + r;
-#pragma unroll
-                for (int t = 0; t < NG; t++) G[t] = __ldcs(gp + t * P);
-#pragma unroll
-                for (int i = 0; i < 2; i++) {
-                    const int o = i * P + q1;
-                    U[i][0] = U[i][1] = 0.0;
-#pragma unroll
-                    for (int b = 0; b < n; b++) {
-                        U[i][0] = fma(v2[b], ad[o + n * b], U[i][0]);
-                        U[i][1] = fma(d2[b], av[o + n * b], U[i][1]);
-                    }
-#pragma unroll
-                    for (int j = 0; j < 2; j++) gu[i][j] = fma(U[i][0], G[j], U[i][1] * G[2 + j]);
-                }
-                s = G[4] * density(gu, A.lam, A.mu);
-            }
-            // the lanes' sum in the cell's first lane, in a fixed order
-            if constexpr (GL == 9) {
-                const double x = __shfl_sync(kFull, s, min(base + 8, 31));
-                if (r == 0) s += x;
-            }
-#pragma unroll
-            for (int o = GL == 16 ? 8 : 4; o > 0; o >>= 1)
-                s += __shfl_sync(kFull, s, min(base + ((r + o) & (GL == 16 ? 15 : 7)), 31));
-        } else {
-            double *const bvv = ad + D * P, *const bvd = bvv + D * P, *const bdv = bvd + D * P;
-            // second index, at (q1, q2, b3)
-#pragma unroll
-            for (int p = 0; p < NP; p++)
-                if (on)
-#pragma unroll
-                    for (int i = 0; i < D; i++) {
-                        const int o = i * P + r + GL * p;
-                        double vv = 0.0, vd = 0.0, dv = 0.0;
-#pragma unroll
-                        for (int b = 0; b < n; b++) {
-                            const double x = av[o + n * (b - q2)], y = ad[o + n * (b - q2)];
-                            vv = fma(v2[b], x, vv);
-                            vd = fma(d2[b], x, vd);
-                            dv = fma(v2[b], y, dv);
-                        }
-                        bvv[o] = vv;
-                        bvd[o] = vd;
-                        bdv[o] = dv;
-                    }
+        double mys = 0.0;   // of cell c0 + lane
+        for (int j = 0; j < A.rounds && c0 + j * NC < A.nc; j++) {
+            const int64_t e = c0 + j * NC + gi;
+            const bool on = gi < NC && e < A.nc;
             __syncwarp();
-            // third index at the points, and the energy there
             if (on)
 #pragma unroll
                 for (int p = 0; p < NP; p++) {
-                    const double *gp = reinterpret_cast<const double *>(A.geo) + e * P * NG + r + GL * p;
-                    double G[NG], gu[D][D];
+                    const int64_t nd = __ldg(A.cell_node + e * P + r + GL * p);
+#pragma unroll
+                    for (int i = 0; i < D; i++) us[i * P + lat[p]] = __ldg(A.u + D * nd + i);
+                }
+            __syncwarp();
+            // first index: av, ad at (q1, b2, b3) = sum_b1 l, l'_(b1)(q1) u(b1, b2, b3)
+            if (on)
+#pragma unroll
+                for (int p = 0; p < NP; p++)
+#pragma unroll
+                    for (int i = 0; i < D; i++) {
+                        const int o = i * P + r + GL * p;
+                        double sv = 0.0, sd = 0.0;
+#pragma unroll
+                        for (int b = 0; b < n; b++) {
+                            const double x = us[o - q1 + b];
+                            sv = fma(v1[b], x, sv);
+                            sd = fma(d1[b], x, sd);
+                        }
+                        av[o] = sv;
+                        ad[o] = sd;
+                    }
+            __syncwarp();
+            double s = 0.0;
+            if constexpr (D == 2) {
+                if (on) {
+                    double U[2][2], gu[2][2], G[NG];
+                    const double *gp = reinterpret_cast<const double *>(A.geo) + e * P * NG + r;
 #pragma unroll
                     for (int t = 0; t < NG; t++) G[t] = __ldcs(gp + t * P);
 #pragma unroll
-                    for (int i = 0; i < D; i++) {
-                        const int o = i * P + q1 + n * q2;
-                        double U[D] = {};
+                    for (int i = 0; i < 2; i++) {
+                        const int o = i * P + q1;
+                        U[i][0] = U[i][1] = 0.0;
 #pragma unroll
                         for (int b = 0; b < n; b++) {
-                            U[0] = fma(v3[p][b], bdv[o + n * n * b], U[0]);
-                            U[1] = fma(v3[p][b], bvd[o + n * n * b], U[1]);
-                            U[2] = fma(d3[p][b], bvv[o + n * n * b], U[2]);
+                            U[i][0] = fma(v2[b], ad[o + n * b], U[i][0]);
+                            U[i][1] = fma(d2[b], av[o + n * b], U[i][1]);
                         }
 #pragma unroll
-                        for (int j = 0; j < D; j++) gu[i][j] = fma(U[0], G[j], fma(U[1], G[3 + j], U[2] * G[6 + j]));
+                        for (int j = 0; j < 2; j++) gu[i][j] = fma(U[i][0], G[j], U[i][1] * G[2 + j]);
                     }
-                    s = fma(G[9], density(gu, A.lam, A.mu), s);
+                    s = G[4] * density(gu, A.lam, A.mu);
                 }
-            s = warp_sum(s);
+                // the lanes' sum in the cell's first lane, in a fixed order
+                if constexpr (GL == 9) {
+                    const double x = __shfl_sync(kFull, s, min(base + 8, 31));
+                    if (r == 0) s += x;
+                }
+#pragma unroll
+                for (int o = GL == 16 ? 8 : 4; o > 0; o >>= 1)
+                    s += __shfl_sync(kFull, s, min(base + ((r + o) & (GL == 16 ? 15 : 7)), 31));
+            } else {
+                double *const bvv = ad + D * P, *const bvd = bvv + D * P, *const bdv = bvd + D * P;
+                // second index, at (q1, q2, b3)
+#pragma unroll
+                for (int p = 0; p < NP; p++)
+                    if (on)
+#pragma unroll
+                        for (int i = 0; i < D; i++) {
+                            const int o = i * P + r + GL * p;
+                            double vv = 0.0, vd = 0.0, dv = 0.0;
+#pragma unroll
+                            for (int b = 0; b < n; b++) {
+                                const double x = av[o + n * (b - q2)], y = ad[o + n * (b - q2)];
+                                vv = fma(v2[b], x, vv);
+                                vd = fma(d2[b], x, vd);
+                                dv = fma(v2[b], y, dv);
+                            }
+                            bvv[o] = vv;
+                            bvd[o] = vd;
+                            bdv[o] = dv;
+                        }
+                __syncwarp();
+                // third index at the points, and the energy there
+                if (on)
+#pragma unroll
+                    for (int p = 0; p < NP; p++) {
+                        const double *gp = reinterpret_cast<const double *>(A.geo) + e * P * NG + r + GL * p;
+                        double G[NG], gu[D][D];
+#pragma unroll
+                        for (int t = 0; t < NG; t++) G[t] = __ldcs(gp + t * P);
+#pragma unroll
+                        for (int i = 0; i < D; i++) {
+                            const int o = i * P + q1 + n * q2;
+                            double U[D] = {};
+#pragma unroll
+                            for (int b = 0; b < n; b++) {
+                                U[0] = fma(v3[p][b], bdv[o + n * n * b], U[0]);
+                                U[1] = fma(v3[p][b], bvd[o + n * n * b], U[1]);
+                                U[2] = fma(d3[p][b], bvv[o + n * n * b], U[2]);
+                            }
+#pragma unroll
+                            for (int j = 0; j < D; j++) gu[i][j] = fma(U[0], G[j], fma(U[1], G[3 + j], U[2] * G[6 + j]));
+                        }
+                        s = fma(G[9], density(gu, A.lam, A.mu), s);
+                    }
+                s = warp_sum(s);
+            }
+            const double x = __shfl_sync(kFull, s, lane % NC * GL);
+            if (lane / NC == j) mys = x;
         }
-        const double x = __shfl_sync(kFull, s, lane % NC * GL);
-        if (lane / NC == j) mys = x;
-      }
-      if (lane < take && c0 + lane < A.nc) put_cell(A, c0 + lane, g, mys, mine);
+        if (lane < take && c0 + lane < A.nc) put_cell(A, c0 + lane, g, mys, mine);
     }
     if (A.c) grid_sum_last_block(mine, A.partial, A.counter, A.c);
 }
