@@ -319,17 +319,22 @@ cudaError_t launch_step(const soptx_mesh_s &m, const double *rho, const double *
         // CTAs take the rest of the GPU and, as those blocks finish, their slots.
         // Blocks per SM, step us: P3 triangles 400x200 FP64 281 at one, 239 at four
         // (the float-pair sensitivity outlasted the assembly at one), FP32 172 / 176;
-        // P2 tets 60x20x20 FP64 364 / 340, FP32 233 / 224.  General quadrilaterals, assembled
+        // P2 tets 60x20x20 FP64 364 / 340, FP32 233 / 224.  Linear cells on FP32 pairs, 25 M
+        // values at one, two, three and four: triangles' step 316 / 181 / 155 / 158 and
+        // backward 750 / 451 / 355 / 318 (their sensitivities outlasted the assembly), sheared
+        // quadrilaterals' 180 / 124 / 128 / 140 and 355 / 247 / 255 / 260; P2 triangles' step
+        // 115 at one and 130 at four.  General quadrilaterals, assembled
         // by the gather, the same way (but one call after the other in the backward of small
         // meshes, where the events cost more than the overlap gives: 31 and 28 us below
         // 2^18 values; Q1 of 1.5 M values 36 beside it, 48 after)
+        const int per_sm = !m.d.contract || m.h.nb == 3 ? 4 : m.h.nb == 4 ? 2 : 1;
         int dev = 0, sms = 0;
         cudaError_t err = cudaGetDevice(&dev);
         if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (err == cudaSuccess) err = cudaEventRecord(m.d.ev[0], st);
         if (err == cudaSuccess) err = cudaStreamWaitEvent(m.d.side, m.d.ev[0], 0);
         if (err == cudaSuccess)
-            err = launch_strain_sensitivity(m, rho, u, dc, c, gscale, m.d.side, m.d.contract ? sms : 4 * sms);
+            err = launch_strain_sensitivity(m, rho, u, dc, c, gscale, m.d.side, per_sm * sms);
         if (err == cudaSuccess) err = cudaEventRecord(m.d.ev[1], m.d.side);
         if (err == cudaSuccess) err = launch_assemble(m, rho, vals, st);
         if (err == cudaSuccess) err = cudaStreamWaitEvent(st, m.d.ev[1], 0);
